@@ -146,8 +146,9 @@ void derive(tclbm_lattice* L) {
     d.inv_Pr = (float)(1.0 / p.Pr);
     d.Pr_m1 = (float)(p.Pr - 1.0);
     d.force_kind = p.force_kind;
-    d.ax = (float)p.ax;
-    d.ay = (float)p.ay;
+    // zero without a uniform acceleration, so that instances which know no other force read none
+    d.ax = p.force_kind == TCLBM_FORCE_ACCEL ? (float)p.ax : 0.0f;
+    d.ay = p.force_kind == TCLBM_FORCE_ACCEL ? (float)p.ay : 0.0f;
     d.famp = (float)p.famp;
     d.rounding = p.storage != TCLBM_STORE_FP32 && p.rounding == TCLBM_ROUND_STOCHASTIC;
     for (int s = 0; s < 4; ++s) {

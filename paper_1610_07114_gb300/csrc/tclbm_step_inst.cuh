@@ -15,18 +15,18 @@ static cudaError_t allow_smem(K kernel, size_t bytes) {
 
 // CTAs of tclbm_step_tile<BX, BY> the current device holds resident at once (0 if the
 // query fails).
-template <int BX, int BY, bool LATE>
+template <int BX, int BY, bool FAST, bool LATE>
 static long long tile_wave() {
     int dev = 0, sms = 0, per_sm = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, tclbm_step_tile<BX, BY, ST, LATE>, BX * BY, 0)) {
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, tclbm_step_tile<BX, BY, ST, FAST, LATE>, BX * BY, 0)) {
         cudaGetLastError();
         return 0;
     }
     return (long long)sms * per_sm;
 }
 
-template <int BX, int BY>
+template <int BX, int BY, bool FAST = false>
 static cudaError_t launch_tile_shape(const DevParams& p, const ST* in, ST* out, cudaStream_t s) {
     // programmatic dependent launch: the next step's grid is scheduled while this one
     // runs (the kernel waits for its predecessor before touching memory); 32 x 4 tiles
@@ -42,13 +42,13 @@ static cudaError_t launch_tile_shape(const DevParams& p, const ST* in, ST* out, 
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     if constexpr (BX == 32 && BY == 4) {
-        static const long long wave = tile_wave<BX, BY, true>();
+        static const long long wave = tile_wave<BX, BY, FAST, true>();
         if (wave > 0 && (long long)cfg.gridDim.x * cfg.gridDim.y > wave) {
-            const cudaError_t e = cudaLaunchKernelEx(&cfg, tclbm_step_tile<BX, BY, ST, true>, p, in, out);
+            const cudaError_t e = cudaLaunchKernelEx(&cfg, tclbm_step_tile<BX, BY, ST, FAST, true>, p, in, out);
             return e != cudaSuccess ? e : cudaGetLastError();
         }
     }
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, tclbm_step_tile<BX, BY, ST, false>, p, in, out);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, tclbm_step_tile<BX, BY, ST, FAST, false>, p, in, out);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
@@ -60,7 +60,8 @@ static cudaError_t launch_tile(int bx, int by, const DevParams& p, const ST* in,
     if (bx == 64 && by == 4) return launch_tile_shape<64, 4>(p, in, out, s);
     if (bx == 64 && by == 8) return launch_tile_shape<64, 8>(p, in, out, s);
     if (bx == 128 && by == 4) return launch_tile_shape<128, 4>(p, in, out, s);
-    return launch_tile_shape<32, 4>(p, in, out, s);
+    // the default shape also comes without the options a lattice does not use
+    return options_fast(p) ? launch_tile_shape<32, 4, true>(p, in, out, s) : launch_tile_shape<32, 4>(p, in, out, s);
 }
 
 // One launch of a TMA-fed step kernel (signature of tclbm_step_tma_corr / _plain) under the
@@ -119,7 +120,9 @@ static cudaError_t launch_tx(const StepLaunch& k, const DevParams& p0, const voi
         cudaError_t e;
         if (corr) {
             static const long long resident = (long long)sm_count() * (CorrShape<ST>::kThreadsPerSM / TX);
-            e = launch_tma(tclbm_step_tma_corr<TX, ST>, TX, tma_smem_bytes<TX, true, ST>(true), resident, k, p, in, out, s);
+            const size_t smem = tma_smem_bytes<TX, true, ST>(true);
+            e = options_fast(p) ? launch_tma(tclbm_step_tma_corr<TX, ST, true>, TX, smem, resident, k, p, in, out, s)
+                                : launch_tma(tclbm_step_tma_corr<TX, ST, false>, TX, smem, resident, k, p, in, out, s);
         } else if (k.thermal) {
             e = launch_tma(tclbm_step_tma_plain<TX, true, ST>, TX, tma_smem_bytes<TX, true, ST>(false),
                            plain_resident<TX, true>(), k, p, in, out, s);
@@ -143,7 +146,8 @@ static cudaError_t launch_tx(const StepLaunch& k, const DevParams& p0, const voi
 
 template <int TX>
 static cudaError_t prepare_tx() {
-    cudaError_t e = allow_smem(tclbm_step_tma_corr<TX, ST>, tma_smem_bytes<TX, true, ST>(true));
+    cudaError_t e = allow_smem(tclbm_step_tma_corr<TX, ST, false>, tma_smem_bytes<TX, true, ST>(true));
+    if (e == cudaSuccess) e = allow_smem(tclbm_step_tma_corr<TX, ST, true>, tma_smem_bytes<TX, true, ST>(true));
     if (e == cudaSuccess) e = allow_smem(tclbm_step_batch_tma<TX, ST>, tma_smem_bytes<TX, true, ST>(true));
     if (e == cudaSuccess) e = allow_smem(tclbm_step_tma_plain<TX, true, ST>, tma_smem_bytes<TX, true, ST>(false));
     if (e == cudaSuccess) e = allow_smem(tclbm_step_tma_plain<TX, false, ST>, tma_smem_bytes<TX, false, ST>(false));

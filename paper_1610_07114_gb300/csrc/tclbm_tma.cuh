@@ -354,7 +354,7 @@ struct CorrShape {
 // kernel parameter or a shared-memory copy; `map` the source copy's tensor map (in
 // parameter or global memory); `smem` the dynamic shared memory of tma_smem_bytes().
 // Returns false after a bounded wait expired (the error word is then set).
-template <int TX, class ST>
+template <int TX, class ST, bool FAST>
 __device__ __forceinline__ bool tma_corr_strip(const DevParams& p, const CUtensorMap* map, const ST* __restrict__ src,
                                                ST* __restrict__ dst, int x0, int y0, int y1, int* __restrict__ err,
                                                unsigned char* smem) {
@@ -408,7 +408,7 @@ __device__ __forceinline__ bool tma_corr_strip(const DevParams& p, const CUtenso
         if (own_valid) {
             float f[9], h[9];
             load_node_ring<TX, true, ST>(p, R, sl, xi, xown, yr, row_wall || col_wall_own, f, h);
-            m = macro_of<true>(p, f, h, xown, yr);
+            m = macro_of<true, FAST>(p, f, h, xown, yr);
 #pragma unroll
             for (int q = 0; q < 9; ++q) {
                 fk[q] = f[q];
@@ -420,7 +420,7 @@ __device__ __forceinline__ bool tma_corr_strip(const DevParams& p, const CUtenso
         if (hslot >= 0 && h_valid) {
             float f[9], h[9];
             load_node_ring<TX, true, ST>(p, R, sl, xih, xh, yr, row_wall || col_wall_halo, f, h);
-            phix[buf][hslot] = phi_x(macro_of<true>(p, f, h, xh, yr));
+            phix[buf][hslot] = phi_x(macro_of<true, FAST>(p, f, h, xh, yr));
         }
     };
     auto phiy_row = [&](int t, int yr, int st) -> float {
@@ -429,7 +429,7 @@ __device__ __forceinline__ bool tma_corr_strip(const DevParams& p, const CUtenso
         const bool row_wall = ywall && (t == 0 || t == ny - 1);
         float f[9], h[9];
         load_node_ring<TX, true, ST>(p, R, sl, xi, xown, yr, row_wall || col_wall_own, f, h);
-        return phi_y(macro_of<true>(p, f, h, xown, yr));
+        return phi_y(macro_of<true, FAST>(p, f, h, xown, yr));
     };
     auto next_slot = [](int st) { return st == RR::NS - 1 ? 0 : st + 1; };
     auto prev_slot = [](int st) { return st == 0 ? RR::NS - 1 : st - 1; };
@@ -476,7 +476,7 @@ __device__ __forceinline__ bool tma_corr_strip(const DevParams& p, const CUtenso
             else
                 dyv = 0.5f * (py_p1 - py_m1);
             float fo[9], ho[9];
-            collide<true>(p, fc, hc, mc, dxv, dyv, fo, ho);
+            collide<true, FAST>(p, fc, hc, mc, dxv, dyv, fo, ho);
             store_node<ST>(p, dst, xl, r, fo, ho, true);
         }
         if (__syncthreads_or(!ok)) {
@@ -583,7 +583,7 @@ __device__ __forceinline__ void seg_mark_done(unsigned* __restrict__ seg_done, u
 
 // seg_done: completion tickets of the work items (nullptr: none published); chain: wait
 // for the neighbouring items of launch ticket - 1 instead of the whole previous grid.
-template <int TX, class ST>
+template <int TX, class ST, bool FAST>
 __global__ void __launch_bounds__(TX, CorrShape<ST>::kThreadsPerSM / TX) tclbm_step_tma_corr(const __grid_constant__ DevParams p, const __grid_constant__ CUtensorMap map,
                                                           const ST* __restrict__ src, ST* __restrict__ dst,
                                                           int rows_per_cta, int seg_full, int seg_extra,
@@ -599,7 +599,7 @@ __global__ void __launch_bounds__(TX, CorrShape<ST>::kThreadsPerSM / TX) tclbm_s
     int y0, y1;
     tma_segment(p, rows_per_cta, seg_full, seg_extra, y0, y1);
     if (chain && !seg_wait_neighbours(p, seg_done, ticket - 1u, err)) return;
-    if (!tma_corr_strip<TX, ST>(p, &map, src, dst, blockIdx.x * TX, y0, y1, err, smem)) return;
+    if (!tma_corr_strip<TX, ST, FAST>(p, &map, src, dst, blockIdx.x * TX, y0, y1, err, smem)) return;
     if (seg_done) seg_mark_done(seg_done, ticket);
     if (blockIdx.x == 0 && blockIdx.y == 0) bump_step_counter(p);
 }
@@ -634,7 +634,9 @@ __global__ void __launch_bounds__(TX, CorrShape<ST>::kThreadsPerSM / TX) tclbm_s
     if (threadIdx.x == 0) asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(map) : "memory");
     const ST* src = static_cast<const ST*>(L->buf[par]);
     ST* dst = static_cast<ST*>(const_cast<void*>(L->buf[par ^ 1]));
-    if (!tma_corr_strip<TX, ST>(sp, map, src, dst, it.x0, it.y0, it.y1, L->err, smem)) return;
+    if (options_fast(sp) ? !tma_corr_strip<TX, ST, true>(sp, map, src, dst, it.x0, it.y0, it.y1, L->err, smem)
+                         : !tma_corr_strip<TX, ST, false>(sp, map, src, dst, it.x0, it.y0, it.y1, L->err, smem))
+        return;
     if (it.x0 == 0 && it.y0 == 0) bump_step_counter(sp);
 }
 

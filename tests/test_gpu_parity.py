@@ -589,3 +589,25 @@ def test_work_term_matches_oracle(T, name, make):
         lat.close()
         print(name, kernel, e)
         assert e["rho"] <= REL_L2 and e["u"] <= REL_L2 and e["T"] <= REL_L2, (name, kernel, e)
+
+
+@pytest.mark.parametrize("storage,rounding", [("fp32", "nearest"), ("fp16", "stochastic"), ("bf16", "nearest")])
+@pytest.mark.parametrize("kernel", [0, 1, 2])
+@pytest.mark.parametrize("nx,ny,walls", [(150, 45, None), (131, 40, ("y", "zouhe")), (70, 32, ("y", "nee"))])
+def test_instances_without_options_equal_the_general_ones(T, nx, ny, walls, kernel, storage, rounding):
+    # a lattice without a force, with constant nu and given rates runs the instance of the
+    # kernel that knows no other option; a Taylor-Green force of zero amplitude is the same
+    # problem on the general instance: bit for bit
+    case, fields = W.random_periodic(nx, ny, seed=91, force="none", storage=storage)
+    if walls:
+        case, fields = W.with_walls(case, fields, axis=walls[0], kind=walls[1])
+    case = dict(case, rounding=rounding)
+    states = []
+    for force in ("none", "taylor_green"):
+        lat = T.Lattice(dict(case, force={"kind": force, "ax": 0.0, "ay": 0.0, "amp": 0.0}), fields)
+        lat.set_kernel(kernel)
+        lat.step(25)
+        states.append(lat.populations())
+        lat.close()
+    (fa, ha), (fb, hb) = states
+    assert np.array_equal(fa, fb) and np.array_equal(ha, hb)
