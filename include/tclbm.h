@@ -124,7 +124,8 @@ typedef struct tclbm_lattice tclbm_lattice;
 /* Number of doubles written by tclbm_diagnostics(). */
 #define TCLBM_NDIAG 8
 
-/* Device bytes one lattice of these parameters holds (state, tables, scratch). */
+/* Device bytes one lattice of these parameters holds (state, tables, scratch), without what
+ * is allocated on first use: the velocity snapshot and the exchange board of tclbm_step(). */
 size_t tclbm_state_bytes(const tclbm_params* params);
 
 /* Validate params, derive constants, allocate the state on the current device.
@@ -146,7 +147,15 @@ tclbm_status tclbm_init_fields(tclbm_lattice* lat, const double* rho, const doub
  * overlap on the device; the first launch of a call waits for whatever precedes it on
  * the stream.  The states are bit-identical to one step per call.  A chained wait that
  * expires is reported like the other bounded waits (TCLBM_ETIMEOUT at the next
- * synchronising call). */
+ * synchronising call).
+ *
+ * A lattice small enough for the shared memory of the device (about 60,000 nodes with the
+ * correction term, 190,000 without, 390,000 athermal; no work term) whose kernel and
+ * launch shape are the library's choice takes 8 or more steps in cooperative launches that
+ * keep its state resident (up to 4096 steps each), unless the stream is capturing.  The
+ * states are the same bit for bit.  The first such call allocates, through the hooks, an
+ * exchange board of 192 bytes per node (96 athermal); without it the lattice takes one
+ * launch per step.  The bounded waits of these launches are reported in the same way. */
 tclbm_status tclbm_step(tclbm_lattice* lat, int64_t nsteps);
 
 /* Macroscopic fields of the current state (Eq. 20; T per Section IV, T0 if athermal),
@@ -221,7 +230,8 @@ const char* tclbm_describe(const tclbm_lattice* lat);
 
 /* Test hook for the timeout path (no counterpart in the paper): with row in [0, ny) the
  * TMA-fed kernel (variant 0, FP32 storage; other formats ignore the hook) never copies
- * that source row, so the bounded waits on it
+ * that source row, and a resident run of tclbm_step() never publishes it to the tiles
+ * around its own, so the bounded waits on it
  * expire after 1 s, the kernel records the failure and returns, and the next
  * synchronising call returns TCLBM_ETIMEOUT (the state is then invalid; re-initialise
  * it).  row = -1 turns the hook off.  EINVAL for other rows. */

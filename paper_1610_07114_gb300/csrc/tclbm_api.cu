@@ -528,6 +528,78 @@ tclbm_status launch_steps(tclbm_lattice* L, int64_t n) {
     return TCLBM_OK;
 }
 
+// Steps of one resident launch at most (a few milliseconds), and the fewest steps worth one:
+// filling and emptying the shared memory costs about as much as two steps.
+constexpr int64_t kResMaxSteps = 4096, kResMinSteps = 8;
+
+int res_kind(const tclbm_params& p) { return !p.thermal ? RES_ATHERMAL : (p.correction ? RES_CORR : RES_THERMAL); }
+
+// Whether L runs resident where enough steps are asked for (planned on first use).
+bool resident_planned(tclbm_lattice* L) {
+    if (!L->auto_kernel || L->dp.work) return false;
+    if (L->res_state == 0) {
+        int dev = 0, coop = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess) {
+            cudaGetLastError();
+            coop = 0;
+        }
+        L->res_state = coop && res_plan(L->dp, res_kind(L->prm), sm_count(), L->res_plan) ? 1 : -1;
+    }
+    return L->res_state > 0;
+}
+
+// Advances L by as many of n steps as resident launches take (`done`); 0 where they do not
+// apply: a kernel or shape chosen by the caller, a lattice too large, the work term (whose
+// rounding differs between the one-step kernels), a capturing stream (a replayed launch
+// would reuse its step numbers), no memory for the board.
+tclbm_status resident_steps(tclbm_lattice* L, int64_t n, int64_t& done) {
+    done = 0;
+    if (n < kResMinSteps || !resident_planned(L)) return TCLBM_OK;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(L->stream, &cap) != cudaSuccess) {
+        cudaGetLastError();
+        return TCLBM_OK;
+    }
+    if (cap != cudaStreamCaptureStatusNone) return TCLBM_OK;
+    if (!L->board) {
+        L->board_bytes = 2 * (size_t)L->prm.nx * L->prm.ny * (size_t)(L->nplanes / 3) * 16;
+        L->board = dev_alloc(L, L->board_bytes);
+        if (!L->board) {
+            L->res_state = -1;
+            return TCLBM_OK;
+        }
+        L->res_tag = 0xffffffffu;  // cleared below
+    }
+    while (n - done >= kResMinSteps) {
+        const int64_t k = n - done < kResMaxSteps ? n - done : kResMaxSteps;
+        if (L->res_tag > 0xffffffffu - (unsigned)k) {  // step numbers start over on a cleared board
+            CK(cudaMemsetAsync(L->board, 0, L->board_bytes, L->stream));
+            L->res_tag = 0;
+        }
+        ResLaunch r;
+        r.plan = L->res_plan;
+        r.kind = res_kind(L->prm);
+        r.parity = L->cur;
+        r.n = (int)k;
+        r.tag0 = L->res_tag;
+        r.board = L->board;
+        r.err = L->err;
+        const cudaError_t e = launch_resident(L->prm.storage, r, L->dp, L->buf[L->cur], L->buf[L->cur ^ 1], L->stream);
+        if (e == cudaErrorCooperativeLaunchTooLarge) {  // fewer multiprocessors than the device has are ours
+            cudaGetLastError();
+            L->res_state = -1;
+            return TCLBM_OK;
+        }
+        if (e != cudaSuccess) return cuda_fail(e, "resident kernel launch");
+        L->res_tag += (unsigned)k;
+        L->cur ^= 1;
+        L->steps += k;
+        done += k;
+    }
+    return TCLBM_OK;
+}
+
 tclbm_status build_graph(tclbm_lattice* L) {
     if (L->graph && L->graph_tx == L->tx && L->graph_ty == L->ty && L->graph_kernel == L->kernel) return TCLBM_OK;
     if (L->kernel == KERNEL_TMA) {
@@ -736,6 +808,7 @@ tclbm_status tclbm_destroy(tclbm_lattice* L) {
     dev_free(L, L->stage, L->stage_bytes);
     dev_free(L, L->err, 256);
     dev_free(L, L->seg_done, L->seg_bytes);
+    dev_free(L, L->board, L->board_bytes);
     if (L->copy_event) cudaEventDestroy(L->copy_event);
     delete L;
     return TCLBM_OK;
@@ -763,6 +836,7 @@ tclbm_status tclbm_set_tile(tclbm_lattice* L, int32_t tx, int32_t ty) {
     }
     L->tx = ntx;
     L->ty = nty;
+    if (tx || ty) L->auto_kernel = false;
     return TCLBM_OK;
 }
 
@@ -806,6 +880,7 @@ tclbm_status tclbm_set_kernel(tclbm_lattice* L, int32_t kind) {
                     kTileBX, kTileBY);
     if (kind != L->kernel) default_shape(L->prm, kind, L->tx, L->ty);
     L->kernel = kind;
+    L->auto_kernel = false;
     return TCLBM_OK;
 }
 
@@ -813,6 +888,11 @@ const char* tclbm_describe(const tclbm_lattice* L) {
     if (!L) return "";
     tclbm_lattice* M = const_cast<tclbm_lattice*>(L);
     describe_step_kernel(L->prm.storage, step_launch(M, 0), L->dp, M->desc, sizeof M->desc);
+    if (resident_planned(M)) {
+        const size_t n = strlen(M->desc);
+        snprintf(M->desc + n, sizeof M->desc - n, "; %d steps or more: tclbm_resident grid (%d, %d) block (%d)",
+                 (int)kResMinSteps, L->res_plan.gx, L->res_plan.gy, L->res_plan.threads);
+    }
     return L->desc;
 }
 
@@ -851,6 +931,12 @@ tclbm_status tclbm_step(tclbm_lattice* L, int64_t nsteps) {
     if (!L) return fail(TCLBM_EINVAL, "lattice is NULL");
     if (nsteps < 0) return fail(TCLBM_EINVAL, "nsteps must be >= 0");
     int64_t left = nsteps;
+    {
+        int64_t done = 0;
+        const tclbm_status st = resident_steps(L, left, done);
+        if (st != TCLBM_OK) return st;
+        left -= done;
+    }
     // long runs of short launches go through a captured graph of 2*kGraphPairs steps
     const long long nodes = (long long)L->prm.nx * L->prm.ny;
     if (left >= 2 * kGraphPairs && nodes <= (1LL << 22)) {

@@ -49,6 +49,15 @@ struct tclbm_lattice {
     unsigned* seg_done = nullptr;
     size_t seg_bytes = 0;
     unsigned ticket = 0;
+    // resident runs (tclbm_resident.cuh): whether the library picks the kernel and its
+    // shape, the plan of this lattice, its exchange board (allocated on first use) and the
+    // number of the last state a run has used
+    bool auto_kernel = true;
+    int res_state = 0;  // 0 not planned yet, 1 planned, -1 does not apply
+    tclbm::ResPlan res_plan{};
+    void* board = nullptr;
+    size_t board_bytes = 0;
+    unsigned res_tag = 0;
     char desc[256] = "";
     // CUDA graph of 2 * kGraphPairs step launches (parity preserved)
     cudaGraphExec_t graph = nullptr;

@@ -8,6 +8,7 @@
 
 #include "tclbm_batch.cuh"
 #include "tclbm_device.cuh"
+#include "tclbm_resident.cuh"
 
 namespace tclbm {
 // Sets the thread-local message returned by tclbm_last_error().
@@ -81,6 +82,62 @@ inline int batch_ctas_per_sm(int storage, int tx, int kind) {
 cudaError_t prepare_step_fp32();
 cudaError_t prepare_step_bf16();
 cudaError_t prepare_step_fp16();
+
+// Resident run of n steps (tclbm_resident.cuh) from `src` to `dst` under `plan`.
+struct ResLaunch {
+    ResPlan plan;
+    int kind;  // RES_*
+    int parity, n;
+    unsigned tag0;
+    void* board;
+    int* err;
+};
+cudaError_t launch_resident_fp32(const ResLaunch& r, const DevParams& p, const void* src, void* dst, cudaStream_t s);
+cudaError_t launch_resident_bf16(const ResLaunch& r, const DevParams& p, const void* src, void* dst, cudaStream_t s);
+cudaError_t launch_resident_fp16(const ResLaunch& r, const DevParams& p, const void* src, void* dst, cudaStream_t s);
+inline cudaError_t launch_resident(int storage, const ResLaunch& r, const DevParams& p, const void* src, void* dst,
+                                   cudaStream_t s) {
+    switch (storage) {
+        case 0: return launch_resident_fp32(r, p, src, dst, s);
+        case 1: return launch_resident_bf16(r, p, src, dst, s);
+        default: return launch_resident_fp16(r, p, src, dst, s);
+    }
+}
+
+// Tiles of a resident run on `sms` CTAs (false: the lattice does not fit).  A CTA takes at
+// least kResMinNodes nodes: below that a step is all latency and more CTAs only add halo.
+constexpr int kResMinNodes = 96;
+inline bool res_plan(const DevParams& p, int kind, int sms, ResPlan& best) {
+    const int R = kind == RES_CORR ? 2 : 1;
+    const long long N = (long long)p.nx * p.ny;
+    const int most_cells = kind == RES_ATHERMAL ? ResShape<RES_ATHERMAL, true>::CELLS : ResShape<RES_CORR, true>::CELLS;
+    if (N > (long long)most_cells * sms) return false;
+    long long most = N / kResMinNodes;
+    most = most < 1 ? 1 : (most > sms ? sms : most);
+    double least = 1e30;
+    for (int gx = 1; gx <= most && gx <= p.nx; ++gx) {
+        long long gy = most / gx;
+        if (gy > p.ny) gy = p.ny;
+        const int bw = (p.nx + gx - 1) / gx, bh = (int)((p.ny + gy - 1) / gy);
+        const int lw = p.nx / gx, lh = (int)(p.ny / gy);  // the smallest tile
+        // a wall's one-sided derivative reads two nodes inside the tile; a halo reaches the next tile only
+        if ((!p.xper && lw < 3) || (!p.yper && lh < 3) || (gx > 1 && lw < R) || (gy > 1 && lh < R)) continue;
+        const bool selfx = gx == 1 && p.xper, selfy = gy == 1 && p.yper;
+        const int own = bw * bh;
+        const int halo = kind == RES_CORR ? (selfx ? 0 : 2 * bh) + (selfy ? 0 : 2 * bw) : 0;
+        const int cells = (bw + 2 * R) * (bh + 2 * R);
+        if (cells - own > 512 || cells > most_cells) continue;
+        const bool multi = own + halo > 512 || cells > 640;
+        if (multi && kind == RES_CORR) continue;  // one launch per step of 2-D tiles is faster there (512 x 256: 5.9 against 7.1 us)
+        const double cost = (multi ? 1.3 : 1.0) * own + 0.4 * halo;
+        if (cost < least) {
+            least = cost;
+            const int threads = multi ? 512 : (own + halo + 31) / 32 * 32;
+            best = ResPlan{gx, (int)gy, threads, multi};
+        }
+    }
+    return least < 1e30;
+}
 
 inline cudaError_t launch_step_kernel(int storage, const StepLaunch& k, const DevParams& p, const void* src,
                                       void* dst, cudaStream_t s) {

@@ -9,4 +9,5 @@ using ST = __half;
 #define BATCH_OCC_FN batch_occupancy_fp16
 #define BATCH_TMA_FN launch_batch_tma_fp16
 #define TMA_RESIDENT_FN tma_resident_fp16
+#define RESIDENT_FN launch_resident_fp16
 #include "tclbm_step_inst.cuh"

@@ -82,6 +82,30 @@ def test_expired_wait_in_a_chain_of_launches_is_reported_and_the_context_recover
     assert np.array_equal(f, f_ref) and np.array_equal(h, h_ref)
 
 
+def test_expired_wait_of_a_resident_run_is_reported_and_the_context_recovers(T):
+    # row 12 is the edge of a tile that never publishes it: the tiles around wait 1 s, set
+    # the error word and return, and so do the others
+    case, fields = W.couette(8, 64)
+    ref = T.Lattice(case, fields)
+    ref.step(20)
+    f_ref, h_ref = ref.populations()
+    ref.close()
+
+    lat = T.Lattice(case, fields)
+    assert "tclbm_resident" in lat.describe()
+    T.tclbm_test_skip_row(lat.handle, 12)
+    lat.step(20)
+    with pytest.raises(T.TclbmError) as err:
+        lat.diagnostics()
+    assert err.value.status == T.ETIMEOUT
+    T.tclbm_test_skip_row(lat.handle, -1)
+    lat.init_fields(fields)
+    lat.step(20)
+    f, h = lat.populations()
+    lat.close()
+    assert np.array_equal(f, f_ref) and np.array_equal(h, h_ref)
+
+
 def test_allocator_returning_null_gives_enomem(T):
     case, _ = W.random_periodic(64, 32, seed=1)
     params = T.params_from_case(case)

@@ -611,3 +611,53 @@ def test_instances_without_options_equal_the_general_ones(T, nx, ny, walls, kern
         lat.close()
     (fa, ha), (fb, hb) = states
     assert np.array_equal(fa, fb) and np.array_equal(ha, hb)
+
+
+def _tg(n, **kw):
+    return W.taylor_green(n, F0=1e-6, nu=0.02, **kw)
+
+
+RESIDENT_CASES = [
+    # tiles that wrap onto themselves on one or both axes, down to one node
+    ("periodic_1x5", lambda: W.random_periodic(1, 5, seed=92)),
+    ("periodic_2x2", lambda: W.random_periodic(2, 2, seed=93)),
+    ("periodic_131x7", lambda: W.random_periodic(131, 7, seed=94)),
+    # walls next to tile edges, three-row and three-column tiles
+    ("ywalls_3x3", lambda: W.with_walls(*W.random_periodic(3, 3, seed=95), axis="y", kind="nee")),
+    ("xwalls_5x3", lambda: W.with_walls(*W.random_periodic(5, 3, seed=96), axis="x", kind="zouhe")),
+    ("ywalls_97x66", lambda: W.with_walls(*W.random_periodic(97, 66, seed=97), axis="y", kind="zouhe")),
+    ("xwalls_100x51", lambda: W.with_walls(*W.random_periodic(100, 51, seed=98), axis="x", kind="equilibrium")),
+    ("couette_8x64", lambda: W.couette(8, 64)),
+    # one node per thread up to the limit of 512 threads, polling with one lane per warp
+    ("rb_300x200", lambda: W.rayleigh_benard(300, 200, seed=99, amp=1e-2)),
+    # more nodes than threads (no correction term); athermal
+    ("thermal_401x399", lambda: W.random_periodic(401, 399, seed=100, correction=False)),
+    ("athermal_64", lambda: _tg(64)),
+    ("athermal_600", lambda: _tg(600)),
+]
+
+
+@pytest.mark.parametrize("storage,rounding", [("fp32", "nearest"), ("fp16", "stochastic"), ("bf16", "nearest")])
+@pytest.mark.parametrize("name,make", RESIDENT_CASES, ids=[c[0] for c in RESIDENT_CASES])
+def test_resident_runs_equal_one_launch_per_step(T, name, make, storage, rounding):
+    # many steps in one launch with the state in shared memory, entered at both parities of
+    # the copies and mixed with single steps, against the one-step kernels: bit for bit
+    case, fields = make()
+    case = dict(case, storage=storage, rounding=rounding)
+    states = []
+    for resident in (True, False):
+        lat = T.Lattice(case, fields)
+        desc = lat.describe()
+        assert "tclbm_resident" in desc, desc
+        if not resident:
+            lat.set_kernel(2 if desc.startswith("tclbm_step_tile") else 1)
+            assert "tclbm_resident" not in lat.describe()
+        for n in (9, 8, 1, 21, 3, 12):
+            lat.step(n)
+        assert lat.steps_done == 54
+        assert np.isfinite(lat.diagnostics()).all()
+        states.append(lat.populations())
+        lat.close()
+    (fa, ha), (fb, hb) = states
+    assert np.array_equal(fa, fb)
+    assert not case["thermal"] or np.array_equal(ha, hb)
