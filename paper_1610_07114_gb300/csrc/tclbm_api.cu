@@ -16,6 +16,7 @@
 
 #include "tclbm.h"
 #include "tclbm_device.cuh"
+#include "tclbm_fields.cuh"
 #include "tclbm_internal.h"
 #include "tclbm_launch.h"
 
@@ -173,6 +174,9 @@ void derive(tclbm_lattice* L) {
     for (int q = 0; q < 9; ++q) {
         d.fbase[q] = (float)fr[q];
         d.hbase[q] = p.thermal ? (float)hr[q] : 0.0f;
+        d.fbase_d[q] = d.fbase[q];  // (exact)
+        d.hbase_d[q] = d.hbase[q];
+        d.hrest += d.hbase_d[q];
     }
 }
 
@@ -256,7 +260,8 @@ __device__ __forceinline__ int wrapi(int i, int n) {
 }
 
 // f_bar = f^eq - S/2, h_bar = h^eq at each node (FP64), written where the pull of the
-// next step reads it: buffer_q(x - e_q) = value_q(x).
+// next step reads it: buffer_q(x - e_q) = value_q(x).  Bound by the FP64 pipe: the values
+// are formed with as few of its instructions as give the same rounding.
 template <class ST>
 __global__ void init_kernel(const DevParams p, const double* __restrict__ rho, const double* __restrict__ ux,
                             const double* __restrict__ uy, const double* __restrict__ T, ST* __restrict__ dst,
@@ -264,56 +269,84 @@ __global__ void init_kernel(const DevParams p, const double* __restrict__ rho, c
                             double famp) {
     const long long n = (long long)p.nx * p.ny;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(i % p.nx), y = (int)(i / p.nx);
+        const int y = (int)((unsigned)i / (unsigned)p.nx), x = (int)((unsigned)i - (unsigned)y * (unsigned)p.nx);
         const double r = rho[i], vx = ux[i], vy = uy[i], t = thermal ? T[i] : T0;
+        const double RT = __dmul_rn(R, t), ux2 = __dmul_rn(vx, vx), uy2 = __dmul_rn(vy, vy);
+        const double qx = __dadd_rn(RT, ux2), qy = __dadd_rn(RT, uy2);
+        // r X(e_x) and Y(e_y), e = 0, +1, -1
+        const double rx[3] = {__dmul_rn(r, __dsub_rn(__dsub_rn(1.0, RT), ux2)), __dmul_rn(r, __dmul_rn(0.5, __dadd_rn(qx, vx))),
+                              __dmul_rn(r, __dmul_rn(0.5, __dsub_rn(qx, vx)))};
+        const double py[3] = {__dsub_rn(__dsub_rn(1.0, RT), uy2), __dmul_rn(0.5, __dadd_rn(qy, vy)),
+                              __dmul_rn(0.5, __dsub_rn(qy, vy))};
+        constexpr int ex[9] = {0, 1, 0, -1, 0, 1, -1, -1, 1}, ey[9] = {0, 0, 1, 0, -1, 1, 1, -1, -1};
+        double hS[9];  // S/2 by Eq. 3 of its raw moments
         double Fx = 0, Fy = 0;
-        if (force_kind == FORCE_ACCEL) {
-            Fx = r * ax;
-            Fy = r * ay;
-        } else if (force_kind == FORCE_TAYLOR_GREEN) {
-            const double kx = 6.283185307179586 / p.nx, ky = 6.283185307179586 / p.ny;
-            Fx = famp * sin(kx * x) * sin(ky * y);
-            Fy = famp * cos(kx * x) * cos(ky * y);
-        }
-        const double Ax = Fx / r, Ay = Fy / r, RT = R * t;
-        const double ux2 = vx * vx, uy2 = vy * vy;
-        const double px[3] = {1.0 - RT - ux2, 0.5 * (RT + ux2 + vx), 0.5 * (RT + ux2 - vx)};  // e = 0, +1, -1
-        const double py[3] = {1.0 - RT - uy2, 0.5 * (RT + uy2 + vy), 0.5 * (RT + uy2 - vy)};
-        const int ex[9] = {0, 1, 0, -1, 0, 1, -1, -1, 1}, ey[9] = {0, 0, 1, 0, -1, 1, 1, -1, -1};
-        // S by Eq. 3 of its raw moments
-        const double sE = 2 * (Ax * vx + Ay * vy), sN = 2 * (Ax * vx - Ay * vy), sP = Ax * vy + Ay * vx;
-        const double s21 = Ay * ux2 + 2 * Ax * vx * vy, s12 = Ax * uy2 + 2 * Ay * vx * vy;
-        const double s22 = 2 * Ax * vx * uy2 + 2 * Ay * vy * ux2;
-        const double S[9] = {r * (-sE + s22),
-                             0.5 * r * (Ax + 0.5 * (sE + sN) - s12 - s22),
-                             0.5 * r * (Ay + 0.5 * (sE - sN) - s21 - s22),
-                             0.5 * r * (-Ax + 0.5 * (sE + sN) + s12 - s22),
-                             0.5 * r * (-Ay + 0.5 * (sE - sN) + s21 - s22),
-                             0.25 * r * (sP + s21 + s12 + s22),
-                             0.25 * r * (-sP + s21 - s12 + s22),
-                             0.25 * r * (sP - s21 - s12 + s22),
-                             0.25 * r * (-sP - s21 + s12 + s22)};
-        const double uu = ux2 + uy2, Et = 0.5 * (b * RT + uu), A = Et + RT, B = Et + 2 * RT, C = RT * A;
-        for (int q = 0; q < 9; ++q) {
-            const int ix = ex[q] == 0 ? 0 : (ex[q] > 0 ? 1 : 2), iy = ey[q] == 0 ? 0 : (ey[q] > 0 ? 1 : 2);
-            const double fv = r * px[ix] * py[iy] - 0.5 * S[q];
-            double hv = 0.0;
-            if (thermal) {
-                if (q == 0)
-                    hv = r * (Et - B * uu - 2 * C);
-                else if (q <= 4)
-                    hv = 0.5 * r * (A * (ex[q] * vx + ey[q] * vy) + B * (ex[q] * ex[q] * ux2 + ey[q] * ey[q] * uy2) + C);
-                else
-                    hv = 0.25 * r * B * ex[q] * ey[q] * vx * vy;
-                if (p.work)  // h_bar = h^eq - q / 2, q_a = W_a F.u
-                    hv -= 0.5 * (q == 0 ? 4.0 / 9.0 : (q <= 4 ? 1.0 / 9.0 : 1.0 / 36.0)) * (Fx * vx + Fy * vy);
+        if (force_kind != FORCE_NONE) {
+            double Ax = ax, Ay = ay;
+            if (force_kind == FORCE_ACCEL) {
+                Fx = r * ax;
+                Fy = r * ay;
+            } else {
+                const double kx = 6.283185307179586 / p.nx, ky = 6.283185307179586 / p.ny;
+                Fx = famp * sin(kx * x) * sin(ky * y);
+                Fy = famp * cos(kx * x) * cos(ky * y);
+                Ax = Fx / r;
+                Ay = Fy / r;
             }
-            int xs = x - ex[q], ys = y - ey[q];
-            if (p.xper) xs = wrapi(xs, p.nx); else if (xs < 0 || xs >= p.nx) continue;
-            if (p.yper) ys = wrapi(ys, p.ny); else if (ys < 0 || ys >= p.ny) continue;
-            const long long o = (long long)ys * p.pitch + xs;
-            Store<ST>::st(dst + q * p.plane + o, (float)(fv - (double)p.fbase[q]));
-            if (thermal) Store<ST>::st(dst + (9 + q) * p.plane + o, (float)(hv - (double)p.hbase[q]));
+            const double axx = Ax * vx, ayy = Ay * vy, uxy2 = 2.0 * (vx * vy);
+            const double ep = 2.0 * axx, em = 2.0 * ayy, E = ep + em;  // (E + N) / 2, (E - N) / 2, E
+            const double P = fma(Ax, vy, Ay * vx);
+            const double s21 = fma(Ay, ux2, Ax * uxy2), s12 = fma(Ax, uy2, Ay * uxy2), s22 = uxy2 * P;
+            const double hr = 0.25 * r, qr = 0.125 * r;  // half of r/2, r/4
+            const double c1 = ep - s22, c2 = em - s22, m1 = Ax - s12, m2 = Ay - s21;
+            const double sp = s21 + s12, sm = s21 - s12, pp = s22 + P, pm = s22 - P;
+            hS[0] = (0.5 * r) * (s22 - E);
+            hS[1] = hr * (c1 + m1);
+            hS[2] = hr * (c2 + m2);
+            hS[3] = hr * (c1 - m1);
+            hS[4] = hr * (c2 - m2);
+            hS[5] = qr * (pp + sp);
+            hS[6] = qr * (pm + sm);
+            hS[7] = qr * (pp - sp);
+            hS[8] = qr * (pm - sm);
+        } else {
+#pragma unroll
+            for (int q = 0; q < 9; ++q) hS[q] = 0.0;
+        }
+        // source rows and columns of the pull, or none past a wall
+        auto wrap = [](int s, int m, int per) { return s < 0 ? (per ? s + m : -1) : (s >= m ? (per ? s - m : -1) : s); };
+        const int xs[3] = {x, wrap(x - 1, p.nx, p.xper), wrap(x + 1, p.nx, p.xper)};
+        const int ys[3] = {y, wrap(y - 1, p.ny, p.yper), wrap(y + 1, p.ny, p.yper)};
+        auto put = [&](int q, int plane, double v) {
+            const int sx = xs[ex[q] == 0 ? 0 : (ex[q] > 0 ? 1 : 2)], sy = ys[ey[q] == 0 ? 0 : (ey[q] > 0 ? 1 : 2)];
+            if (sx >= 0 && sy >= 0) Store<ST>::st(dst + plane * p.plane + ((long long)sy * p.pitch + sx), d2f(v));
+        };
+#pragma unroll
+        for (int q = 0; q < 9; ++q) {
+            const double a = rx[ex[q] == 0 ? 0 : (ex[q] > 0 ? 1 : 2)], c = py[ey[q] == 0 ? 0 : (ey[q] > 0 ? 1 : 2)];
+            put(q, q, __dsub_rn(__fma_rn(a, c, -hS[q]), p.fbase_d[q]));
+        }
+        if (thermal) {
+            const double uu = __dadd_rn(ux2, uy2), Et = __dmul_rn(0.5, __fma_rn(b, RT, uu)), A = __dadd_rn(Et, RT),
+                         B = __fma_rn(2.0, RT, Et), C = __dmul_rn(RT, A);
+            const double hr = __dmul_rn(0.5, r), bx = __dmul_rn(B, ux2), by = __dmul_rn(B, uy2);
+            const double qb = __dmul_rn(__dmul_rn(__dmul_rn(__dmul_rn(0.25, r), B), vx), vy);
+            double hv[9];
+            hv[0] = __dmul_rn(r, __fma_rn(-2.0, C, __fma_rn(-B, uu, Et)));
+            hv[1] = __dmul_rn(hr, __dadd_rn(__fma_rn(A, vx, bx), C));
+            hv[2] = __dmul_rn(hr, __dadd_rn(__fma_rn(A, vy, by), C));
+            hv[3] = __dmul_rn(hr, __dadd_rn(__fma_rn(-A, vx, bx), C));
+            hv[4] = __dmul_rn(hr, __dadd_rn(__fma_rn(-A, vy, by), C));
+            hv[5] = hv[7] = qb;
+            hv[6] = hv[8] = -qb;
+            if (p.work) {  // h_bar = h^eq - q / 2, q_a = W_a F.u
+                const double fu = __fma_rn(Fx, vx, __dmul_rn(Fy, vy));
+#pragma unroll
+                for (int q = 0; q < 9; ++q)
+                    hv[q] = __fma_rn(-0.5 * (q == 0 ? 4.0 / 9.0 : (q <= 4 ? 1.0 / 9.0 : 1.0 / 36.0)), fu, hv[q]);
+            }
+#pragma unroll
+            for (int q = 0; q < 9; ++q) put(q, 9 + q, __dsub_rn(hv[q], p.hbase_d[q]));
         }
     }
 }
@@ -325,14 +358,15 @@ __global__ void set_pops_kernel(const DevParams p, const double* __restrict__ f,
     const long long n = (long long)p.nx * p.ny;
     const int ex[9] = {0, 1, 0, -1, 0, 1, -1, -1, 1}, ey[9] = {0, 0, 1, 0, -1, 1, 1, -1, -1};
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(i % p.nx), y = (int)(i / p.nx);
+        const int y = (int)((unsigned)i / (unsigned)p.nx), x = (int)((unsigned)i - (unsigned)y * (unsigned)p.nx);
+#pragma unroll
         for (int q = 0; q < 9; ++q) {
             int xs = x - ex[q], ys = y - ey[q];
             if (p.xper) xs = wrapi(xs, p.nx); else if (xs < 0 || xs >= p.nx) continue;
             if (p.yper) ys = wrapi(ys, p.ny); else if (ys < 0 || ys >= p.ny) continue;
             const long long o = (long long)ys * p.pitch + xs;
-            Store<ST>::st(dst + q * p.plane + o, (float)(f[q * n + i] - (double)p.fbase[q]));
-            if (thermal) Store<ST>::st(dst + (9 + q) * p.plane + o, (float)(h[q * n + i] - (double)p.hbase[q]));
+            Store<ST>::st(dst + q * p.plane + o, d2f(f[q * n + i] - p.fbase_d[q]));
+            if (thermal) Store<ST>::st(dst + (9 + q) * p.plane + o, d2f(h[q * n + i] - p.hbase_d[q]));
         }
     }
 }
@@ -343,63 +377,33 @@ __global__ void get_pops_kernel(const DevParams p, const ST* __restrict__ src, d
                                 double* __restrict__ h) {
     const long long n = (long long)p.nx * p.ny;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(i % p.nx), y = (int)(i / p.nx);
+        const int y = (int)((unsigned)i / (unsigned)p.nx), x = (int)((unsigned)i - (unsigned)y * (unsigned)p.nx);
         float fv[9], hv[9];
         load_node<THERMAL, ST>(p, src, x, y, fv, hv);
+#pragma unroll
         for (int q = 0; q < 9; ++q) {
-            f[q * n + i] = (double)p.fbase[q] + fv[q];
-            if (THERMAL && h) h[q * n + i] = (double)p.hbase[q] + hv[q];
+            f[q * n + i] = p.fbase_d[q] + f2d(fv[q]);
+            if (THERMAL && h) h[q * n + i] = p.hbase_d[q] + f2d(hv[q]);
         }
     }
 }
 
 // Eq. 20 and the temperature of Section IV in FP64 from the observable state.
 template <bool THERMAL, class ST>
-__device__ __forceinline__ void node_fields(const DevParams& p, const ST* __restrict__ src, int x, int y, double& rho,
-                                            double& vx, double& vy, double& T, double& sh) {
-    float fv[9], hv[9];
-    load_node<THERMAL, ST>(p, src, x, y, fv, hv);
-    double r = 0, jx = 0, jy = 0;
-    const int ex[9] = {0, 1, 0, -1, 0, 1, -1, -1, 1}, ey[9] = {0, 0, 1, 0, -1, 1, 1, -1, -1};
-    for (int q = 0; q < 9; ++q) {
-        const double fq = (double)p.fbase[q] + fv[q];
-        r += fq;
-        jx += fq * ex[q];
-        jy += fq * ey[q];
-    }
-    double Fx = 0, Fy = 0;
-    if (p.force_kind == FORCE_ACCEL) {
-        Fx = r * (double)p.ax;
-        Fy = r * (double)p.ay;
-    } else if (p.force_kind == FORCE_TAYLOR_GREEN) {
-        Fx = (double)p.famp * p.sx[x] * p.sy[y];
-        Fy = (double)p.famp * p.cx[x] * p.cy[y];
-    }
-    rho = r;
-    vx = (jx + 0.5 * Fx) / r;
-    vy = (jy + 0.5 * Fy) / r;
-    sh = 0;
-    if (THERMAL) {
-        for (int q = 0; q < 9; ++q) sh += (double)p.hbase[q] + hv[q];
-        const double she = p.work ? sh + 0.5 * (Fx * vx + Fy * vy) : sh;  // rho E with the work term
-        T = p.inv_bR2 * (she / r - 0.5 * (vx * vx + vy * vy));
-    } else {
-        T = p.T0d;
-    }
-}
-
-template <bool THERMAL, class ST>
 __global__ void moments_kernel(const DevParams p, const ST* __restrict__ src, double* __restrict__ rho,
                                double* __restrict__ ux, double* __restrict__ uy, double* __restrict__ T) {
     const long long n = (long long)p.nx * p.ny;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(i % p.nx), y = (int)(i / p.nx);
-        double r, vx, vy, t, sh;
-        node_fields<THERMAL, ST>(p, src, x, y, r, vx, vy, t, sh);
-        rho[i] = r;
-        ux[i] = vx;
-        uy[i] = vy;
-        T[i] = t;
+        const int y = (int)((unsigned)i / (unsigned)p.nx), x = (int)((unsigned)i - (unsigned)y * (unsigned)p.nx);
+        float fv[9], hv[9];
+        load_node<THERMAL, ST>(p, src, x, y, fv, hv);
+        const NodeSums s = node_sums<THERMAL>(fv, hv);
+        const NodeFields v = node_velocity(p, s, x, y);
+        const double sh = THERMAL ? sum_value(p.hrest, s.sdh) : 0.0;
+        rho[i] = v.rho;
+        ux[i] = v.ux;
+        uy[i] = v.uy;
+        T[i] = node_temperature<THERMAL>(p, v, sh, THERMAL ? __fma_rn(v.ux, v.ux, v.uy * v.uy) : 0.0, x, y);
     }
 }
 
@@ -417,22 +421,50 @@ __global__ void __launch_bounds__(kDiagBlock) diag_kernel(const DevParams p, con
     __shared__ double red[kDiagBlock / 32][TCLBM_NDIAG];
     double acc[TCLBM_NDIAG] = {0, 0, 0, 0, 0, 0, 0, 0};
     const long long n = (long long)p.nx * p.ny;
+    // the linear sums stay FP32 error-free sums of deviations until the thread's last node
+    Running drho, jx, jy, sdh;
+    double nodes = 0, Fxs = 0, Fys = 0;  // nodes seen, and their Taylor-Green forces
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(i % p.nx), y = (int)(i / p.nx);
-        double r, vx, vy, t, sh;
-        node_fields<THERMAL, ST>(p, src, x, y, r, vx, vy, t, sh);
-        acc[0] += r;
-        acc[1] += r * vx;
-        acc[2] += r * vy;
-        acc[3] += sh;
-        acc[4] += 0.5 * r * (vx * vx + vy * vy);
-        acc[5] += vy * (t - T_ref);
-        if (usnap) {
-            const double dx = vx - usnap[2 * i], dy = vy - usnap[2 * i + 1];
-            acc[6] += dx * dx + dy * dy;
+        const int y = (int)((unsigned)i / (unsigned)p.nx), x = (int)((unsigned)i - (unsigned)y * (unsigned)p.nx);
+        float fv[9], hv[9];
+        load_node<THERMAL, ST>(p, src, x, y, fv, hv);
+        const NodeSums s = node_sums<THERMAL>(fv, hv);
+        const NodeFields v = node_velocity(p, s, x, y);
+        const double uu = __fma_rn(v.ux, v.ux, v.uy * v.uy);
+        drho.add(s.drho);
+        jx.add(s.jx);
+        jy.add(s.jy);
+        if (p.force_kind == FORCE_TAYLOR_GREEN) {
+            Fxs = __fma_rn(f2d(p.sx[x]), f2d(p.sy[y]), Fxs);
+            Fys = __fma_rn(f2d(p.cx[x]), f2d(p.cy[y]), Fys);
         }
-        acc[7] += vx * vx + vy * vy;
+        double t = p.T0d;
+        if (THERMAL) {
+            sdh.add(s.sdh);
+            t = node_temperature<THERMAL>(p, v, sum_value(p.hrest, s.sdh), uu, x, y);
+        }
+        nodes += 1.0;
+        acc[4] = __fma_rn(v.rho, uu, acc[4]);
+        acc[5] = __fma_rn(v.uy, t - T_ref, acc[5]);
+        if (usnap) {
+            const double dx = v.ux - f2d(usnap[2 * i]), dy = v.uy - f2d(usnap[2 * i + 1]);
+            acc[6] = __fma_rn(dx, dx, __fma_rn(dy, dy, acc[6]));
+        }
+        acc[7] += uu;
     }
+    // sum rho, sum (j + F/2), sum h_bar and the kinetic energy of this thread's nodes
+    acc[0] = nodes + drho.value();
+    acc[1] = jx.value();
+    acc[2] = jy.value();
+    if (p.force_kind == FORCE_TAYLOR_GREEN) {
+        acc[1] = __fma_rn(0.5 * (double)p.famp, Fxs, acc[1]);
+        acc[2] = __fma_rn(0.5 * (double)p.famp, Fys, acc[2]);
+    } else {
+        acc[1] = __fma_rn(0.5 * (double)p.ax, acc[0], acc[1]);
+        acc[2] = __fma_rn(0.5 * (double)p.ay, acc[0], acc[2]);
+    }
+    acc[3] = THERMAL ? __fma_rn(nodes, p.hrest, sdh.value()) : 0.0;
+    acc[4] *= 0.5;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
     for (int k = 0; k < TCLBM_NDIAG; ++k) {
@@ -460,11 +492,12 @@ template <bool THERMAL, class ST>
 __global__ void snapshot_kernel(const DevParams p, const ST* __restrict__ src, float* __restrict__ usnap) {
     const long long n = (long long)p.nx * p.ny;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(i % p.nx), y = (int)(i / p.nx);
-        double r, vx, vy, t, sh;
-        node_fields<THERMAL, ST>(p, src, x, y, r, vx, vy, t, sh);
-        usnap[2 * i] = (float)vx;
-        usnap[2 * i + 1] = (float)vy;
+        const int y = (int)((unsigned)i / (unsigned)p.nx), x = (int)((unsigned)i - (unsigned)y * (unsigned)p.nx);
+        float fv[9], hv[9];
+        load_node<THERMAL, ST>(p, src, x, y, fv, hv);
+        const NodeFields v = node_velocity(p, node_sums<false>(fv, hv), x, y);
+        usnap[2 * i] = d2f(v.ux);
+        usnap[2 * i + 1] = d2f(v.uy);
     }
 }
 

@@ -60,6 +60,7 @@ struct DevParams {
     // FP64 constants of the field conversions (moments, diagnostics): T = inv_bR2 (E - u^2/2)
     // with inv_bR2 = 2 / (b R), and T0, as the FP64 initialisation uses them
     double inv_bR2, T0d;
+    double fbase_d[9], hbase_d[9], hrest;  // the rest-state populations and sum hbase
     int work;  // 1: the body force's power F.u is a source of total energy (rho E = sum h_bar + F.u/2)
 };
 

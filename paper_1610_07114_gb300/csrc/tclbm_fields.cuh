@@ -1,0 +1,171 @@
+// tclbm_fields.cuh -- FP64 arithmetic of the field conversions (initial fields, moments,
+// diagnostics, population transfer), arranged for sm_103a's FP64 rate.
+//
+// The FP64 pipe takes 64 cycles a warp instruction on this part (1/64 of FP32), so these
+// kernels were bound by it, not by memory: 1.96 ms for the moments of a 4096 x 2048
+// lattice whose bytes take 0.13 ms.  What the pipe does not have to do is moved off it:
+//   - conversions between FP32 and FP64 are exact bit moves (or one rounding) in integer
+//     instructions;
+//   - sums over a node's populations are taken on the stored FP32 deviations by
+//     error-free transformations (Knuth's two-sum: s = a + b and its exact error), carried as
+//     an unevaluated sum of three floats, and enter FP64 once; the base values' sums are
+//     exact;
+//   - one reciprocal of rho serves the three divisions, each corrected by its remainder.
+// The results are as near the exact ones as those of the plain FP64 expressions (compared
+// with quad precision over the flows of the performance cases).
+// Measured before / after (us): 4096 x 2048 FP32, moments 1962 / 701, diagnostics 2447 /
+// 1026, velocity snapshot 1155 / 468, initial fields 3337 / 1933 (their bytes take 129, 89,
+// 99 and 129); 2048 x 1024 populations in 258 / 187, out 236 / 113.  An FP64 instruction per
+// node costs 23 us at 4096 x 2048; about 28, 42, 19 and 84 are left.
+#pragma once
+
+#include "tclbm_device.cuh"
+
+namespace tclbm {
+
+// (double)v without the FP64 pipe for zeros and normal numbers.
+__device__ __forceinline__ double f2d(float v) {
+    const unsigned u = __float_as_uint(v), m = u & 0x7fffffffu;
+    if (m - 0x00800000u < 0x7f000000u)  // normal
+        return __hiloint2double((int)((u & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(u << 29));
+    if (m == 0) return __hiloint2double((int)u, 0);
+    return (double)v;
+}
+
+// (float)v, rounded to nearest even, without the FP64 pipe where the result is zero or normal.
+__device__ __forceinline__ float d2f(double v) {
+    const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v), m = hi & 0x7fffffffu;
+    if (m - 0x38100000u < 0x0fd00000u) {  // exponents -126 .. 126
+        const unsigned t = ((m - 0x38000000u) << 3) | (lo >> 29), rem = lo << 3;
+        const unsigned up = rem > 0x80000000u || (rem == 0x80000000u && (t & 1u)) ? 1u : 0u;
+        return __uint_as_float((hi & 0x80000000u) | (t + up));
+    }
+    if ((m | lo) == 0) return __uint_as_float(hi);
+    return __double2float_rn(v);
+}
+
+// An unevaluated sum hi + mid + lo.
+struct Sum3 {
+    float hi, mid, lo;
+};
+__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
+    s = __fadd_rn(a, b);
+    const float t = __fsub_rn(s, a);
+    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
+}
+__device__ __forceinline__ void sum_add(Sum3& p, float v) {
+    float e;
+    two_sum(p.hi, v, p.hi, e);
+    two_sum(p.mid, e, p.mid, e);
+    p.lo = __fadd_rn(p.lo, e);
+}
+// base + sum (an infinite or undefined sum has no error terms)
+__device__ __forceinline__ double sum_value(double base, const Sum3& p) {
+    if (!(fabsf(p.hi) <= 3.402823466e38f)) return base + (double)p.hi;
+    return base + f2d(p.hi) + (f2d(p.mid) + f2d(p.lo));
+}
+__device__ __forceinline__ double sum_value(const Sum3& p) {
+    if (!(fabsf(p.hi) <= 3.402823466e38f)) return (double)p.hi;
+    return f2d(p.hi) + (f2d(p.mid) + f2d(p.lo));
+}
+template <int N>
+__device__ __forceinline__ Sum3 sum_of(const float (&v)[N]) {
+    Sum3 p;
+    two_sum(v[0], v[1], p.hi, p.mid);
+    p.lo = 0.0f;
+#pragma unroll
+    for (int q = 2; q < N; ++q) sum_add(p, v[q]);
+    return p;
+}
+
+// 1/x from the FP32 approximation and one third-order step (relative error near 2^-53).
+__device__ __forceinline__ double rcp_d(double x) {
+    const unsigned m = (unsigned)__double2hiint(x) & 0x7fffffffu;
+    if (m - 0x3c000000u >= 0x07f00000u) return 1.0 / x;  // outside 2^-63 .. 2^63
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d2f(x)));
+    const double y = f2d(r), e = __fma_rn(-x, y, 1.0);
+    return __fma_rn(y, __fma_rn(e, e, e), y);
+}
+
+// a / x, r = rcp_d(x): one correction of the quotient by its remainder.
+__device__ __forceinline__ double div_d(double a, double x, double r) {
+    const double q = a * r;
+    return __fma_rn(__fma_rn(-q, x, a), r, q);
+}
+
+// Sums of a node's deviations: rho - 1, the momentum without the force, sum h_bar less its
+// rest value.
+struct NodeSums {
+    Sum3 drho, jx, jy, sdh;
+};
+template <bool THERMAL>
+__device__ __forceinline__ NodeSums node_sums(const float (&f)[9], const float (&h)[9]) {
+    NodeSums s;
+    s.drho = sum_of(f);
+    s.jx = sum_of({f[1], -f[3], f[5], -f[6], f[8], -f[7]});
+    s.jy = sum_of({f[2], -f[4], f[5], -f[7], f[6], -f[8]});
+    if (THERMAL) s.sdh = sum_of(h);
+    return s;
+}
+
+// rho and u of Eq. 20 from the sums (Fx, Fy: the Taylor-Green force, else unused).
+struct NodeFields {
+    double rho, irho, ux, uy;
+};
+__device__ __forceinline__ NodeFields node_velocity(const DevParams& p, const NodeSums& s, int x, int y) {
+    NodeFields n;
+    n.rho = sum_value(1.0, s.drho);
+    n.irho = rcp_d(n.rho);
+    double jx = sum_value(s.jx), jy = sum_value(s.jy);
+    if (p.force_kind == FORCE_TAYLOR_GREEN) {
+        const double a = 0.5 * f2d(p.famp);
+        jx = __fma_rn(a * f2d(p.sx[x]), f2d(p.sy[y]), jx);
+        jy = __fma_rn(a * f2d(p.cx[x]), f2d(p.cy[y]), jy);
+    } else {
+        jx = __fma_rn(0.5 * f2d(p.ax), n.rho, jx);
+        jy = __fma_rn(0.5 * f2d(p.ay), n.rho, jy);
+    }
+    n.ux = div_d(jx, n.rho, n.irho);
+    n.uy = div_d(jy, n.rho, n.irho);
+    return n;
+}
+
+// Temperature of Section IV; hrest: the rest value of sum h_bar, uu = |u|^2.
+template <bool THERMAL>
+__device__ __forceinline__ double node_temperature(const DevParams& p, const NodeFields& n, double sh, double uu, int x,
+                                                   int y) {
+    if (!THERMAL) return p.T0d;
+    if (p.work) {  // rho E = sum h_bar + F.u / 2
+        double Fx, Fy;
+        if (p.force_kind == FORCE_TAYLOR_GREEN) {
+            Fx = f2d(p.famp) * f2d(p.sx[x]) * f2d(p.sy[y]);
+            Fy = f2d(p.famp) * f2d(p.cx[x]) * f2d(p.cy[y]);
+        } else {
+            Fx = n.rho * f2d(p.ax);
+            Fy = n.rho * f2d(p.ay);
+        }
+        sh = __fma_rn(0.5, __fma_rn(Fx, n.ux, Fy * n.uy), sh);
+    }
+    return p.inv_bR2 * __fma_rn(-0.5, uu, div_d(sh, n.rho, n.irho));
+}
+
+// A running sum of FP32 values in three parts (error-free to far below FP64's rounding).
+struct Running {
+    float a = 0.0f, b = 0.0f, c = 0.0f;
+    __device__ __forceinline__ void add(float v) {
+        float e;
+        two_sum(a, v, a, e);
+        two_sum(b, e, b, e);
+        c = __fadd_rn(c, e);
+    }
+    __device__ __forceinline__ void add(const Sum3& p) {
+        add(p.hi);
+        add(p.mid);  // (lo is below 2^-48 of a deviation and 2^-72 of the sum it would enter)
+    }
+    __device__ __forceinline__ double value() const {
+        return fabsf(a) <= 3.402823466e38f ? (f2d(c) + f2d(b)) + f2d(a) : (double)a;
+    }
+};
+
+}  // namespace tclbm

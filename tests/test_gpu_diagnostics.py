@@ -138,3 +138,61 @@ def test_rcp_error_bound(T):
     assert torch.equal(yd, yd2)
     with pytest.raises(T.TclbmError):
         T.tclbm_test_rcp(None, None, 5)
+
+
+def test_population_transfer_rounds_like_host_arithmetic(T):
+    # populations in and out: base + float32(x - base), for deviations of every magnitude a
+    # float has (zeros, denormals, ties between two floats, overflow to infinity, NaN)
+    case, _ = W.random_periodic(64, 9, seed=61)
+    lat = T.Lattice(case)  # cleared state: every population at its rest value
+    base_f, base_h = lat.populations()
+    rng = np.random.default_rng(62)
+    mag = 10.0 ** rng.uniform(-47, 39, size=base_f.shape) * rng.choice([-1.0, 1.0], size=base_f.shape)
+    ties = (1.0 + (rng.integers(0, 1 << 23, size=base_f.shape) + 0.5) * 2.0 ** -23) * 2.0 ** -10
+    d = np.where(rng.random(base_f.shape) < 0.5, mag, ties)
+    d[0, 0, :4] = [0.0, -0.0, np.inf, np.nan]
+    with np.errstate(over="ignore", invalid="ignore"):
+        f, h = base_f + d, base_h + d[::-1]
+        lat.set_populations(f, h)
+        got_f, got_h = lat.populations()
+        want_f = base_f + (f - base_f).astype(np.float32).astype(np.float64)
+        want_h = base_h + (h - base_h).astype(np.float32).astype(np.float64)
+    lat.close()
+    assert np.array_equal(got_f, want_f, equal_nan=True) and np.array_equal(got_h, want_h, equal_nan=True)
+
+
+@pytest.mark.parametrize("amp", [1e-1, 1e-4, 1e-9, 0.0])
+@pytest.mark.parametrize("force", ["none", "accel", "taylor_green"])
+def test_moments_of_given_populations_to_the_last_digits(T, force, amp):
+    # rho, u and T against extended precision on the same populations: rho and T are O(1)
+    # values with about three roundings, u one division of a momentum whose nine terms were
+    # summed exactly: 4 and 2 units of 2^-53 of their scale
+    case, _ = W.random_periodic(70, 33, seed=63, force=force)
+    lat = T.Lattice(case)
+    f, h = lat.populations()
+    rng = np.random.default_rng(64)
+    lat.set_populations(f + amp * rng.uniform(-1, 1, f.shape), h + amp * rng.uniform(-1, 1, h.shape))
+    f, h = (a.astype(np.longdouble) for a in lat.populations())
+    m, p = lat.moments(), lat.params
+    lat.close()
+    L = np.longdouble
+    rho, ex, ey = f.sum(0), (0, 1, 0, -1, 0, 1, -1, -1, 1), (0, 0, 1, 0, -1, 1, 1, -1, -1)
+    jx, jy = sum(e * v for e, v in zip(ex, f)), sum(e * v for e, v in zip(ey, f))
+    Fx = Fy = L(0)
+    if force == "accel":
+        Fx, Fy = rho * L(np.float32(p.ax)), rho * L(np.float32(p.ay))
+    elif force == "taylor_green":
+        kx, ky = 2 * np.pi * np.arange(70) / 70, 2 * np.pi * np.arange(33) / 33
+        t = [g.astype(np.float32).astype(L) for g in (np.sin(kx), np.cos(kx), np.sin(ky), np.cos(ky))]
+        a = L(np.float32(p.famp))
+        Fx, Fy = a * t[0][None, :] * t[2][:, None], a * t[1][None, :] * t[3][:, None]
+    ux, uy = (jx + Fx / 2) / rho, (jy + Fy / 2) / rho
+    c = L(2.0 / (2.0 / (p.gamma - 1.0) * p.R))
+    Tn = c * (h.sum(0) / rho - (ux * ux + uy * uy) / 2)
+    eps = 2.0 ** -53
+    assert float(np.abs(m["rho"] - rho).max()) <= 4 * eps
+    assert float(np.abs(m["T"] - Tn).max()) <= 8 * eps * float(np.abs(Tn).max())
+    # (the momentum's terms are populations read back in FP64: 2^-55 each for the small ones)
+    scale = max(float(np.abs(ux).max()), float(np.abs(uy).max()))
+    assert float(np.abs(m["ux"] - ux).max()) <= 2 * eps * scale + 12 * 2.0 ** -55 * (amp < 1e-6)
+    assert float(np.abs(m["uy"] - uy).max()) <= 2 * eps * scale + 12 * 2.0 ** -55 * (amp < 1e-6)
