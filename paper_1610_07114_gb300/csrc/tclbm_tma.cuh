@@ -15,8 +15,11 @@
 // registers, so its collision reads no ring row and a slot is free one row after its
 // last lookahead use; the plain kernel pulls at collision time and frees slots later.
 // A launch that finds the error word set returns at once.  Periodic wrap in x: strips whose
-// box crosses x = 0 or x = nx patch the wrapped columns from global memory after the
-// row lands; in y the producer requests the wrapped (or clamped) row directly.
+// box crosses x = 0 or x = nx patch the wrapped columns they read from global memory after
+// the row lands, with values fetched one row ahead: such strips are the slowest ones, and
+// chained launches advance at the pace of their slowest strips (4096 x 2048 FP32 228.3 us a
+// step with the values fetched when the row lands and a barrier of their own, 220.1 so); in
+// y the producer requests the wrapped (or clamped) row directly.
 //
 // Every wait is bounded by the global timer; on expiry the CTA records an error code,
 // drains its own outstanding copies (again bounded) and returns.
@@ -85,6 +88,15 @@ __device__ __forceinline__ void tma_row(void* dst, const CUtensorMap* map, uint6
         : "memory");
 }
 
+// Wrap patches read rows that the previous step's CTAs may have written while this grid was
+// already resident (chained launches): through L2, never the read-only path.
+__device__ __forceinline__ float patch_ld(const float* p) { return __ldcg(p); }
+template <class ST>
+__device__ __forceinline__ ST patch_ld(const ST* p) {
+    const unsigned short u = __ldcg(reinterpret_cast<const unsigned short*>(p));
+    return *reinterpret_cast<const ST*>(&u);
+}
+
 template <class ST>
 struct TmaGeom {
     static constexpr int M = 16 / (int)sizeof(ST);  // halo columns each side; keeps x * size on 16 B
@@ -142,6 +154,29 @@ struct RowRing {
     int freed_to;         // highest source row whose slot was handed back for a refill
     bool patch;           // strip box crosses x = 0 or x = nx on a periodic x axis
     int xb;               // logical column of box index 0
+    // wrapped columns of a patched strip: the three left of x = 0 and the three right of nx - 1
+    // that its nodes read, one value per thread and turn, fetched one row ahead
+    static constexpr int WRAP = 3, TURNS = (2 * WRAP * NP + TX - 1) / TX;
+    ST wrap_v[TURNS];
+    long long wrap_src[TURNS];  // offset in a source row, planes included
+    int wrap_dst[TURNS];        // place in a ring slot (-1: none)
+
+    __device__ __forceinline__ void wrap_setup(const DevParams& p) {
+#pragma unroll
+        for (int t = 0; t < TURNS; ++t) {
+            const int i = (int)threadIdx.x + t * TX, q = i / (2 * WRAP), k = i - q * 2 * WRAP;
+            const int x = k < WRAP ? k - WRAP : p.nx + k - WRAP;  // logical column
+            const int c = x - xb;
+            wrap_dst[t] = q < NP && c >= 0 && c < BOXW ? q * BOXW + c : -1;
+            wrap_src[t] = (long long)q * p.plane + ((x % p.nx) + p.nx) % p.nx;
+        }
+    }
+    __device__ __forceinline__ void wrap_fetch(const DevParams& p, const ST* __restrict__ src, int s) {
+        const ST* row = src + (long long)phys_row(p, s) * p.pitch;
+#pragma unroll
+        for (int t = 0; t < TURNS; ++t)
+            if (wrap_dst[t] >= 0) wrap_v[t] = patch_ld(row + wrap_src[t]);
+    }
 
     __device__ __forceinline__ int slot(int s) const { return (s - s_first) % NS; }
     __device__ __forceinline__ uint32_t parity(int s) const { return (uint32_t)(((s - s_first) / NS) & 1); }
@@ -158,36 +193,25 @@ struct RowRing {
             tma_row(ring + (size_t)slot(s) * SLOT_ELEMS, map, bar + slot(s), xb, phys_row(p, s), ROW_BYTES);
         issued_to = s;
     }
-    // every thread: make sources up to `s_need` available; false on timeout
+    // every thread: make sources up to `s_need` available; false on timeout.  A patched strip
+    // asks for one row more than it reads (ahead()): what a thread patches here is read by
+    // others only after the next barrier.
+    __device__ __forceinline__ int ahead() const { return patch ? 1 : 0; }
     __device__ __forceinline__ bool acquire(const DevParams& p, const ST* __restrict__ src, int s_need) {
         if (s_need > s_last) s_need = s_last;
         bool ok = true;
-        bool patched = false;
         while (ready_to < s_need) {
             const int s = ready_to + 1;
             ok = mbar_wait(bar + slot(s), parity(s)) && ok;
             if (patch) {
-                // wrapped columns of a periodic x axis, straight from global memory: the
-                // box columns left of x = 0 (n_left of them) and right of nx - 1 (n_right)
                 ST* row = ring + (size_t)slot(s) * SLOT_ELEMS;
-                const ST* srow = src + (long long)phys_row(p, s) * p.pitch;
-                const int n_left = xb < 0 ? -xb : 0;
-                const int c_right = p.nx - xb;  // first box column with x >= nx
-                const int n_right = c_right < BOXW ? BOXW - c_right : 0;
-                const int ncol = n_left + n_right;
-                for (int i = threadIdx.x; i < ncol * NP; i += blockDim.x) {
-                    const int q = i / ncol, k = i - q * ncol;
-                    const int c = k < n_left ? k : c_right + (k - n_left);
-                    int xp = xb + c;
-                    xp = xp < 0 ? xp + p.nx : xp - p.nx;
-                    if (xp < 0 || xp >= p.nx) xp = ((xp % p.nx) + p.nx) % p.nx;  // nx smaller than the halo
-                    row[q * BOXW + c] = srow[(long long)q * p.plane + xp];
-                }
-                patched = true;
+#pragma unroll
+                for (int t = 0; t < TURNS; ++t)
+                    if (wrap_dst[t] >= 0) row[wrap_dst[t]] = wrap_v[t];
+                if (s < s_last) wrap_fetch(p, src, s + 1);
             }
             ready_to = s;
         }
-        if (patched) __syncthreads();
         return ok;
     }
     // every thread, after a timeout was agreed on: wait (bounded) for copies still in flight
@@ -238,7 +262,8 @@ __device__ __forceinline__ Slots5 slots_around(int st) {  // st = ring slot of r
 
 template <int TX, bool THERMAL, class ST>
 __device__ __forceinline__ void ring_setup(RowRing<TX, THERMAL, ST>& R, unsigned char* smem, const CUtensorMap* map,
-                                           int x0, int s_first, int s_last, const DevParams& p) {
+                                           const ST* __restrict__ src, int x0, int s_first, int s_last,
+                                           const DevParams& p) {
     using RR = RowRing<TX, THERMAL, ST>;
     R.ring = reinterpret_cast<ST*>(smem);
     R.bar = reinterpret_cast<uint64_t*>(smem + RR::RING_BYTES);  // 8 barrier words reserved
@@ -258,6 +283,10 @@ __device__ __forceinline__ void ring_setup(RowRing<TX, THERMAL, ST>& R, unsigned
     if (threadIdx.x == 0) {
         const int last = s_first + RR::NS - 1 < s_last ? s_first + RR::NS - 1 : s_last;
         for (int s = s_first; s <= last; ++s) R.issue(p, s);
+    }
+    if (R.patch) {
+        R.wrap_setup(p);
+        R.wrap_fetch(p, src, s_first);
     }
 }
 
@@ -312,14 +341,19 @@ __global__ void __launch_bounds__(TX, 512 / TX) tclbm_step_tma_plain(const __gri
     int y0, y1;
     tma_segment(p, rows_per_cta, seg_full, seg_extra, y0, y1);
     // output row r pulls sources r-1..r+1; a wall row's neighbour reaches r-2 / r+2
-    ring_setup<TX, THERMAL, ST>(R, smem, &map, x0, y0 - 2, y1 + 1, p);
+    ring_setup<TX, THERMAL, ST>(R, smem, &map, src, x0, y0 - 2, y1 + 1, p);
     const int x = x0 + tid;
     const bool owns = x < p.nx;
     const int xi = tid + RR::M;
     const bool col_wall = !p.xper && (x == 0 || x == p.nx - 1);
     int st = R.slot(y0);
+    bool ok = true;
+    if (R.patch) {
+        ok = R.acquire(p, src, y0 + 2);
+        __syncthreads();
+    }
     for (int r = y0; r < y1; ++r) {
-        const bool ok = R.acquire(p, src, r + 2);
+        ok = R.acquire(p, src, r + 2 + R.ahead()) && ok;
         if (owns) {
             const Slots5 sl = slots_around<RR::NS>(st);
             const bool maybe_wall = col_wall || (!p.yper && (r == 0 || r == p.ny - 1));
@@ -371,7 +405,7 @@ __device__ __forceinline__ bool tma_corr_strip(const DevParams& p, const CUtenso
     const int s_first = short_top ? y0 - 3 : y0 - 2;
     int s_last = y1 + 1;
     if (ywall && y0 == 0 && s_last < 3) s_last = 3;
-    ring_setup<TX, true, ST>(R, smem, map, x0, s_first, s_last, p);
+    ring_setup<TX, true, ST>(R, smem, map, src, x0, s_first, s_last, p);
 
     const int xl = x0 + tid;  // logical column of this thread
     const bool owns = xl < nx;
@@ -436,7 +470,8 @@ __device__ __forceinline__ bool tma_corr_strip(const DevParams& p, const CUtenso
 
     bool ok = true;
     // prologue: phi_y of row y0-1 (if it exists) and the moments of row y0
-    ok = R.acquire(p, src, y0 + 2) && ok;  // a bottom-wall row y0 reads its neighbour's sources up to y0+2
+    ok = R.acquire(p, src, y0 + 2 + R.ahead()) && ok;  // a bottom-wall row y0 reads its neighbour's sources up to y0+2
+    if (R.patch) __syncthreads();
     int st = R.slot(y0);                    // ring slot of row r (collision row)
     int yr_next = p.yper ? (y0 + 1 == ny ? 0 : y0 + 1) : y0 + 1;  // physical row r + 1
     if (y0 > 0 || p.yper) py_m1 = phiy_row(y0 - 1, y0 == 0 ? ny - 1 : y0 - 1, prev_slot(st));
@@ -454,7 +489,7 @@ __device__ __forceinline__ bool tma_corr_strip(const DevParams& p, const CUtenso
         const int buf_n = buf_c == 2 ? 0 : buf_c + 1;
         int need = r + 2;
         if (ywall && r == 0) need = 3;
-        ok = R.acquire(p, src, need) && ok;
+        ok = R.acquire(p, src, need + R.ahead()) && ok;
         if (has_next) moments_row(r + 1, yr_next, next_slot(st), mn, py_p1, buf_n, fn, hn);
         float py_p2 = 0.f;
         if (ywall && r == 0) py_p2 = phiy_row(2, 2, next_slot(next_slot(st)));
@@ -509,10 +544,11 @@ __device__ __forceinline__ bool tma_corr_strip(const DevParams& p, const CUtenso
 // waiting for the whole previous grid (griddepcontrol.wait), a CTA waits only for the
 // nine work items around its own (strip +-1, segment +-1, wrapped on periodic axes) to
 // have finished the previous step.  Those items wrote every source row this CTA reads
-// (rows y0-3 .. y1+1 and columns x0-M .. x0+TX+M, inside those items where every segment
-// has at least 4 rows and the last strip at least M columns: the host chains only such
+// (rows y0-3 .. y1+1 and columns x0-3 .. x0+TX+2, inside those items where every segment
+// has at least 4 rows and the last strip at least 3 columns: the host chains only such
 // plans) and were the only readers of the rows it overwrites, so the wait covers both
-// orders.  Each item
+// orders.  (The row copies and wrap patches bring up to M columns on each side; the ones past
+// those three are never used, whatever step they are from.)  Each item
 // publishes, once all its stores are issued, the launch's ticket (a per-lattice counter
 // that only grows) in seg_done[blockIdx.y * gridDim.x + blockIdx.x]; the next launch
 // (ticket + 1) proceeds once the nine entries reach ticket.  The next grid is released
