@@ -59,6 +59,10 @@ struct tclbm_batch {
     cudaGraphExec_t graph = nullptr;
     bool graph_valid = false;
     cudaEvent_t ev = nullptr;
+    // streams of the groups beside the first one present, and the events that fork them from
+    // the batch stream and join them again (created where a batch has several groups)
+    cudaStream_t side[3] = {nullptr, nullptr, nullptr};
+    cudaEvent_t fork = nullptr, join[3] = {nullptr, nullptr, nullptr};
     char desc[256] = "";
 };
 
@@ -267,29 +271,49 @@ tclbm_status join_streams(tclbm_batch* B, bool after) {
     return TCLBM_OK;
 }
 
-// One batch step: a launch per kernel group present.
-cudaError_t launch_one_step(const tclbm_batch* B, int parity, cudaStream_t s) {
-    if (B->count[kGroupTma] > 0) {
-        const cudaError_t e = launch_batch_tma_kernel(B->storage, B->tma_tx, B->grid[kGroupTma], B->d_lats,
-                                                      B->d_items + B->first[kGroupTma], B->count[kGroupTma], parity, s);
-        if (e != cudaSuccess) return e;
+// One step of one kernel group.
+cudaError_t launch_group(const tclbm_batch* B, int g, int parity, cudaStream_t s) {
+    if (g == kGroupTma)
+        return launch_batch_tma_kernel(B->storage, B->tma_tx, B->grid[g], B->d_lats, B->d_items + B->first[g], B->count[g],
+                                       parity, s);
+    return launch_batch_kernel(B->storage, B->tx, g, B->grid[g], B->d_lats, B->d_items + B->first[g], B->count[g], parity, s);
+}
+
+// n steps from parity `parity`, ordered on `s`.  The groups hold different lattices, so each
+// runs its own chain of launches beside the others: a group of a few narrow lattices takes
+// about as long as its rows are deep (40 us for 64 x 32 lattices in 16-row strips) and
+// would otherwise leave the device idle once a step.
+tclbm_status launch_chain(tclbm_batch* B, int64_t n, int parity, cudaStream_t s) {
+    int groups[4], ng = 0;
+    for (int g : {kGroupTma, (int)BATCH_THERMAL_CORR, (int)BATCH_THERMAL, (int)BATCH_ATHERMAL})
+        if (B->count[g] > 0) groups[ng++] = g;
+    cudaStream_t on[4] = {s, s, s, s};
+    if (ng > 1) {
+        if (!B->fork) CK(cudaEventCreateWithFlags(&B->fork, cudaEventDisableTiming));
+        CK(cudaEventRecord(B->fork, s));
+        for (int i = 1; i < ng; ++i) {
+            if (!B->side[i - 1]) CK(cudaStreamCreateWithFlags(&B->side[i - 1], cudaStreamNonBlocking));
+            if (!B->join[i - 1]) CK(cudaEventCreateWithFlags(&B->join[i - 1], cudaEventDisableTiming));
+            on[i] = B->side[i - 1];
+            CK(cudaStreamWaitEvent(on[i], B->fork, 0));
+        }
     }
-    for (int k = 2; k >= 0; --k) {
-        if (B->count[k] == 0) continue;
-        const cudaError_t e = launch_batch_kernel(B->storage, B->tx, k, B->grid[k], B->d_lats,
-                                                  B->d_items + B->first[k], B->count[k], parity, s);
-        if (e != cudaSuccess) return e;
+    cudaError_t e = cudaSuccess;
+    for (int64_t k = 0; k < n && e == cudaSuccess; ++k)
+        for (int i = 0; i < ng && e == cudaSuccess; ++i) e = launch_group(B, groups[i], (int)((parity + k) & 1), on[i]);
+    for (int i = 1; i < ng; ++i) {  // also after a failed launch: nothing may outlive the batch stream's order
+        const cudaError_t r = cudaEventRecord(B->join[i - 1], on[i]);
+        const cudaError_t w = r == cudaSuccess ? cudaStreamWaitEvent(s, B->join[i - 1], 0) : r;
+        if (e == cudaSuccess) e = w;
     }
-    return cudaSuccess;
+    return e == cudaSuccess ? TCLBM_OK : cuda_fail(e, "batched step kernel launch");
 }
 
 tclbm_status launch_batch_steps(tclbm_batch* B, int64_t n) {
-    for (int64_t s = 0; s < n; ++s) {
-        const cudaError_t e = launch_one_step(B, (int)(B->steps & 1), B->stream);
-        if (e != cudaSuccess) return cuda_fail(e, "batched step kernel launch");
-        ++B->steps;
-    }
-    return TCLBM_OK;
+    if (n <= 0) return TCLBM_OK;
+    tclbm_status st = launch_chain(B, n, (int)(B->steps & 1), B->stream);
+    if (st == TCLBM_OK) B->steps += n;
+    return st;
 }
 
 tclbm_status build_batch_graph(tclbm_batch* B) {
@@ -302,11 +326,15 @@ tclbm_status build_batch_graph(tclbm_batch* B) {
     CK(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
+    tclbm_status ls = TCLBM_OK;
     if (e == cudaSuccess) {
-        for (int s = 0; s < 2 * kGraphPairs && e == cudaSuccess; ++s)
-            e = launch_one_step(B, s & 1, cs);
-        const cudaError_t e2 = cudaStreamEndCapture(cs, &g);
-        if (e == cudaSuccess) e = e2;
+        ls = launch_chain(B, 2 * kGraphPairs, 0, cs);
+        e = cudaStreamEndCapture(cs, &g);
+    }
+    if (ls != TCLBM_OK) {
+        if (g) cudaGraphDestroy(g);
+        cudaStreamDestroy(cs);
+        return ls;
     }
     if (e == cudaSuccess) e = cudaGraphInstantiate(&B->graph, g, 0);
     if (g) cudaGraphDestroy(g);
@@ -608,6 +636,11 @@ tclbm_status tclbm_batch_destroy(tclbm_batch* B) {
     cudaStreamSynchronize(B->stream);
     if (B->graph) cudaGraphExecDestroy(B->graph);
     if (B->ev) cudaEventDestroy(B->ev);
+    if (B->fork) cudaEventDestroy(B->fork);
+    for (int i = 0; i < 3; ++i) {
+        if (B->join[i]) cudaEventDestroy(B->join[i]);
+        if (B->side[i]) cudaStreamDestroy(B->side[i]);
+    }
     for (auto& st : B->stage) {
         if (st.used) cudaEventDestroy(st.used);
         if (st.host) cudaFreeHost(st.host);
