@@ -184,7 +184,7 @@ void derive(tclbm_lattice* L) {
 // direct-load kernel with short strips where tiles do not apply) expose the most
 // parallelism.  Larger lattices stream rows through the TMA ring with 128-wide strips
 // of 16 or 32 rows per CTA (default_shape).
-constexpr long long kSmallNodes = 1LL << 21;
+constexpr long long kSmallNodes = 1LL << 21, kChainNodes = 1LL << 20;
 
 // Launch shape a kernel variant gets by default: (tx, rows per CTA) for the marching
 // kernels, the tile (BX, BY) for KERNEL_TILE.
@@ -198,35 +198,33 @@ void default_shape(const tclbm_params& p, int kernel, int& tx, int& ty) {
         long long t = (long long)p.ny * strips / (8LL * 152);
         ty = (int)(t < 2 ? 2 : (t > 16 ? 16 : t));
     } else {
-        // 16 rows per CTA, or 32 (fewer halo rows per node) where the last wave's tail
-        // weighs little: where the 32-row grid spans more than two waves of the kernel's
-        // resident CTAs, so its tail of half-height segments applies (ny a multiple of 8),
-        // else where it spans at least 8 waves.  Measured with the short tail: 32 rows tie
-        // 16 at 4096 x 2048 and beat it by 1 % at 2048 x 2048 (FP32) and by 4-5 % at
-        // 8192 x 4096; 16 rows win by 12-20 % where the 32-row grid has no short tail
-        // (FP16 2048 x 2048, athermal 2048 x 2048).
+        // Without the correction term: 16 rows per CTA, or 32 (fewer halo rows per node) where
+        // the last wave's tail weighs little: where the 32-row grid spans more than two waves
+        // of the kernel's resident CTAs, so its tail of half-height segments applies (ny a
+        // multiple of 8), else where it spans at least 8 waves (16 rows win by 12-20 % on
+        // athermal 2048 x 2048, which has no short tail at 32).
         tx = p.nx >= 512 ? 128 : (p.nx >= 96 ? 64 : 32);
         const long long strips = (p.nx + tx - 1) / tx;
         const long long resident = tma_resident(p.storage, tx, p.thermal && p.correction, p.thermal);
-        // Chained launches (tclbm_step: the correction-term kernel, FP32 or 16-bit with
-        // round-to-nearest) overlap consecutive steps, so the tail no longer sets the
-        // segment height: the tallest of 96, 64 and 48 rows whose grid still spans three
-        // waves of resident CTAs (measured against 16-96 rows: 4096 x 2048 FP32 takes 48
-        // rows, 0.722 -> 0.740 of peak; 8192 x 4096 takes 96, FP32 0.738 -> 0.779, FP16
-        // 0.389 -> 0.405); grids that reach three waves at none of them keep the rule below.
-        const bool chained = p.thermal && p.correction &&
-                             (p.storage == TCLBM_STORE_FP32 || p.rounding == TCLBM_ROUND_NEAREST);
-        if (chained) {
+        if (p.thermal && p.correction) {
+            // Chained launches overlap consecutive steps, so the tail no longer sets the
+            // segment height: the tallest segments whose grid spans 1.65 waves of resident
+            // CTAs.  Measured (us per step at 16 / 32 / 48 / 64 rows): 4096 x 2048 FP32 245 /
+            // 227 / 220 / 217 with 9.0 / 4.9 / 3.5 / 2.7 waves, FP16 234 / 218 / 214 / 210 with
+            // 6.8 / 3.8 / 2.7 / 1.7; 2048 x 2048 bf16 120 / 109 / 151 / 130 with 3.4 / 1.7 /
+            // 1.1 / 0.8; 2051 x 1537 FP32 104 / 98 / 101 / 124 with 3.6 / 1.8 / 1.2 / 0.9.
             DevParams d = {};
             d.nx = p.nx;
             d.ny = p.ny;
-            for (int rows : {96, 64, 48}) {
+            for (int rows : {96, 64, 48, 32, 16}) {
                 const SegPlan plan = tma_seg_plan(d, tx, rows, resident);
-                if (strips * (plan.full + plan.half) >= 3 * resident) {
+                if (20 * strips * (plan.full + plan.half) >= 33 * resident) {
                     ty = rows;
                     return;
                 }
             }
+            ty = 8;
+            return;
         }
         if (p.ny % 8 == 0)
             ty = strips * (p.ny / 32) > 2 * resident ? 32 : 16;
@@ -243,7 +241,13 @@ bool tile_fits(const tclbm_params& p, int bx, int by) {
 
 void default_launch(const tclbm_params& p, int& tx, int& ty, int& kernel) {
     const long long n = (long long)p.nx * p.ny;
-    if (n <= kSmallNodes)
+    // With the correction term chained TMA launches take over from the tiles at 2^20 nodes
+    // (us per step, tiles / chained: 2048 x 1024 FP32 81 / 68, FP16 87 / 66; 1024 x 1024 42.5 /
+    // 39; 1024 x 512 19.5 / 26).  The work term, which the tiles round their own way, and
+    // lattices whose last strip is too narrow to chain stay with them up to 2^21.
+    const int tail = p.nx % 128;
+    const bool chains = p.thermal && p.correction && !p.work && (tail == 0 || tail >= 3);
+    if (n <= kSmallNodes && !(chains && n >= kChainNodes && p.nx >= 512))
         kernel = tile_fits(p, kTileBX, kTileBY) ? KERNEL_TILE : KERNEL_DIRECT;
     else
         kernel = KERNEL_TMA;
@@ -479,13 +483,16 @@ __global__ void __launch_bounds__(kDiagBlock) diag_kernel(const DevParams p, con
     }
 }
 
-__global__ void diag_finish(const double* __restrict__ partial, int nblocks, double* __restrict__ out) {
-    const int k = threadIdx.x;
-    if (k < TCLBM_NDIAG) {
-        double s = 0;
-        for (int b = 0; b < nblocks; ++b) s += partial[b * TCLBM_NDIAG + k];
-        out[k] = s;
-    }
+// Warp k sums quantity k over the block partials (a single thread's chain of 1024 additions
+// took 45 us); the error word of the step kernels rides along in out[TCLBM_NDIAG].
+__global__ void diag_finish(const double* __restrict__ partial, int nblocks, const int* __restrict__ err,
+                            double* __restrict__ out) {
+    const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    double s = 0;
+    for (int b = lane; b < nblocks; b += 32) s += partial[b * TCLBM_NDIAG + k];
+    s = warp_sum(s);
+    if (lane == 0) out[k] = s;
+    if (threadIdx.x == 0) out[TCLBM_NDIAG] = (double)*err;
 }
 
 template <bool THERMAL, class ST>
@@ -534,29 +541,48 @@ StepLaunch step_launch(tclbm_lattice* L, int src) {
     return k;
 }
 
+// Whether consecutive TMA launches of L can be chained: the correction-term kernel, row
+// segments of at least 4 rows (half-height tails of 8-row plans), and a last strip at least
+// as wide as the three columns its neighbours read of it.  (The row copies bring more
+// columns than that; what they bring of a strip further away is never used.)
+bool chainable(const tclbm_lattice* L) {
+    const int tail = L->prm.nx % L->tx;
+    return L->kernel == KERNEL_TMA && L->prm.thermal && L->prm.correction && L->ty >= 8 && (tail == 0 || tail >= 3);
+}
+
 tclbm_status launch_steps(tclbm_lattice* L, int64_t n) {
     if (n > 0 && L->kernel == KERNEL_TMA) {
         tclbm_status st = ensure_maps(L);
         if (st != TCLBM_OK) return st;
     }
     // TMA launches with the correction term publish per-item completion tickets; after the
-    // first launch of this run the next one waits for each item's neighbours only (16-bit
-    // stochastic rounding keeps whole-grid waits: its step counter is written by one CTA)
-    const int tx = L->tx, nx = L->prm.nx;
+    // first launch of this run the next one waits for each item's neighbours only
     const bool tickets = L->kernel == KERNEL_TMA && L->prm.thermal && L->prm.correction;
-    const bool chainable = tickets && !L->dp.rounding && L->ty >= 8 && (nx % tx == 0 || nx % tx >= 8);
+    const bool chain = n > 1 && chainable(L);
+    const int first = L->cur;
     for (int64_t s = 0; s < n; ++s) {
         StepLaunch k = step_launch(L, L->cur);
         if (tickets) {
             k.seg_done = L->seg_done;
             k.seg_cap = (long long)(L->seg_bytes / sizeof(unsigned));
             k.ticket = ++L->ticket;
-            k.chain = chainable && s > 0;
+            k.chain = chain && s > 0;
+        }
+        if (chain && L->dp.rounding) {  // no launch of the chain may write the counter others read
+            k.ctr_copy = first;
+            k.ctr_add = (unsigned)s;
         }
         const cudaError_t e = launch_step_kernel(L->prm.storage, k, L->dp, L->buf[L->cur], L->buf[L->cur ^ 1], L->stream);
         if (e != cudaSuccess) return cuda_fail(e, "step kernel launch");
         L->cur ^= 1;
         ++L->steps;
+    }
+    if (chain && L->dp.rounding) {
+        DevParams p = L->dp;
+        p.parity = first;
+        tclbm_count_steps<<<1, 1, 0, L->stream>>>(p, L->cur, (unsigned)n);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return cuda_fail(e, "step counter");
     }
     return TCLBM_OK;
 }
@@ -737,7 +763,7 @@ size_t tclbm_state_bytes(const tclbm_params* p) {
     const size_t planes = p->thermal ? 18 : 9;
     const size_t pops = 2 * planes * (size_t)p->ny * pitch_of(p->nx) * elem_of(p->storage);
     const size_t tables = sizeof(float) * 2 * ((size_t)p->nx + p->ny);
-    const size_t diag = sizeof(double) * (kDiagMaxBlocks + 1) * TCLBM_NDIAG;
+    const size_t diag = sizeof(double) * ((kDiagMaxBlocks + 1) * TCLBM_NDIAG + 1);
     return pops + tables + diag + n * 4 * sizeof(double) + seg_entries(p->nx, p->ny) * sizeof(unsigned);
 }
 
@@ -763,7 +789,7 @@ tclbm_status tclbm_create(const tclbm_params* params, tclbm_alloc_fn alloc, tclb
     const size_t n = (size_t)params->nx * params->ny;
     L->buf_bytes = (size_t)L->nplanes * L->dp.plane * L->elem;
     L->tables_bytes = sizeof(float) * 2 * ((size_t)params->nx + params->ny);
-    L->diag_bytes = sizeof(double) * (kDiagMaxBlocks + 1) * TCLBM_NDIAG;
+    L->diag_bytes = sizeof(double) * ((kDiagMaxBlocks + 1) * TCLBM_NDIAG + 1);
     L->stage_bytes = n * 4 * sizeof(double);
     L->buf[0] = dev_alloc(L, L->buf_bytes);
     L->buf[1] = dev_alloc(L, L->buf_bytes);
@@ -972,7 +998,8 @@ tclbm_status tclbm_step(tclbm_lattice* L, int64_t nsteps) {
     }
     // long runs of short launches go through a captured graph of 2*kGraphPairs steps
     const long long nodes = (long long)L->prm.nx * L->prm.ny;
-    if (left >= 2 * kGraphPairs && nodes <= (1LL << 22)) {
+    // (chained TMA launches overlap on the device, which a graph's whole-grid waits do not)
+    if (left >= 2 * kGraphPairs && nodes <= (1LL << 22) && !chainable(L)) {
         if (L->cur != 0) {
             tclbm_status st = launch_steps(L, 1);
             if (st != TCLBM_OK) return st;
@@ -1012,8 +1039,7 @@ tclbm_status tclbm_moments(tclbm_lattice* L, double* rho, double* ux, double* uy
         for (int k = 0; k < 4; ++k)
             if (out[k])
                 CK(cudaMemcpyAsync(out[k], dst[k], n * sizeof(double), cudaMemcpyDeviceToHost, L->stream));
-    CK(cudaStreamSynchronize(L->stream));
-    return check_kernel_error(L);
+    return check_kernel_error(L);  // synchronises
 }
 
 tclbm_status tclbm_snapshot_velocity(tclbm_lattice* L) {
@@ -1049,15 +1075,16 @@ tclbm_status tclbm_diagnostics(tclbm_lattice* L, double out[TCLBM_NDIAG]) {
             diag_kernel<true, ST><<<(int)nb, kDiagBlock, 0, L->stream>>>(L->dp, src, L->usnap, L->prm.T_ref, L->diag);
         else
             diag_kernel<false, ST><<<(int)nb, kDiagBlock, 0, L->stream>>>(L->dp, src, L->usnap, L->prm.T_ref, L->diag);
-        diag_finish<<<1, 32, 0, L->stream>>>(L->diag, (int)nb, res);
+        diag_finish<<<1, 32 * TCLBM_NDIAG, 0, L->stream>>>(L->diag, (int)nb, L->err, res);
         return TCLBM_OK;
     });
     if (st != TCLBM_OK) return st;
     CK(cudaGetLastError());
-    CK(cudaMemcpyAsync(out, res, TCLBM_NDIAG * sizeof(double), cudaMemcpyDeviceToHost, L->stream));
+    double got[TCLBM_NDIAG + 1];
+    CK(cudaMemcpyAsync(got, res, sizeof got, cudaMemcpyDeviceToHost, L->stream));
     CK(cudaStreamSynchronize(L->stream));
-    tclbm_status ks = check_kernel_error(L);
-    if (ks != TCLBM_OK) return ks;
+    memcpy(out, got, TCLBM_NDIAG * sizeof(double));
+    if (got[TCLBM_NDIAG] != 0.0) return check_kernel_error(L);  // reports and clears it
     for (int k = 0; k < TCLBM_NDIAG; ++k)
         if (!std::isfinite(out[k])) return fail(TCLBM_ENONFINITE, "non-finite diagnostic %d", k);
     return TCLBM_OK;
@@ -1089,7 +1116,7 @@ tclbm_status tclbm_get_populations(tclbm_lattice* L, double* f, double* h, int32
         e = cudaMemcpyAsync(f, df, bytes, cudaMemcpyDeviceToHost, L->stream);
         if (e == cudaSuccess && h && L->prm.thermal) e = cudaMemcpyAsync(h, dh, bytes, cudaMemcpyDeviceToHost, L->stream);
     }
-    if (e == cudaSuccess) e = cudaStreamSynchronize(L->stream);
+    if (e == cudaSuccess && tmp) e = cudaStreamSynchronize(L->stream);
     if (tmp) dev_free(L, tmp, 2 * bytes);
     if (st != TCLBM_OK) return st;
     if (e != cudaSuccess) return cuda_fail(e, "get_populations");

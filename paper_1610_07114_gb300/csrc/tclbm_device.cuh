@@ -55,7 +55,9 @@ struct DevParams {
     float fbase[9], hbase[9];  // rest-state populations f^eq(1, 0, T0), h^eq(1, 0, T0)
     int rounding;              // 16-bit stores: 0 nearest, 1 stochastic
     unsigned* step_ctr;        // two step counters, alternated by launch parity
-    int parity;                // index of the source copy of this launch
+    int parity;                // index of the source copy of this launch (and of its step counter)
+    unsigned ctr_add;          // steps since the counter was written (chained launches leave it alone)
+    int ctr_hold;              // 1: this launch does not advance the counter
     int skip_row;              // test hook: the TMA producer never copies this source row (-1: off)
     // FP64 constants of the field conversions (moments, diagnostics): T = inv_bR2 (E - u^2/2)
     // with inv_bR2 = 2 / (b R), and T0, as the FP64 initialisation uses them
@@ -728,7 +730,7 @@ __device__ __forceinline__ void store_node(const DevParams& p, ST* __restrict__ 
     const long long P = p.plane, o = (long long)y * p.pitch + x;
     if (sizeof(ST) == 2 && p.rounding) {
         // stochastic rounding, two planes per conversion
-        const uint32_t step = p.step_ctr[p.parity];
+        const uint32_t step = p.step_ctr[p.parity] + p.ctr_add;
         const uint32_t node = (uint32_t)(y * p.nx + x);
         const uint32_t seed = sr_bits(node, 0u, step);  // one full mix per node
         float v[18];
@@ -759,7 +761,7 @@ __device__ __forceinline__ void store_node(const DevParams& p, ST* __restrict__ 
 // Advances the stochastic-rounding step counter for the next launch (thread 0 of the
 // one CTA that owns the lattice's first strip and row).
 __device__ __forceinline__ void bump_step_counter(const DevParams& p) {
-    if (p.rounding && threadIdx.x == 0) p.step_ctr[p.parity ^ 1] = p.step_ctr[p.parity] + 1u;
+    if (p.rounding && !p.ctr_hold && threadIdx.x == 0) p.step_ctr[p.parity ^ 1] = p.step_ctr[p.parity] + 1u;
 }
 
 // ---------------------------------------------------------------- the fused step

@@ -31,7 +31,7 @@ struct tclbm_lattice {
     size_t buf_bytes = 0;
     float* tables = nullptr;
     size_t tables_bytes = 0;
-    double* diag = nullptr;  // [kDiagMaxBlocks * TCLBM_NDIAG] partials + TCLBM_NDIAG result
+    double* diag = nullptr;  // [kDiagMaxBlocks * TCLBM_NDIAG] partials + TCLBM_NDIAG + 1 results
     size_t diag_bytes = 0;
     float* usnap = nullptr;  // 2 * nx * ny
     size_t usnap_bytes = 0;

@@ -43,6 +43,10 @@ struct StepLaunch {
     long long seg_cap = 0;
     unsigned ticket = 0;
     int chain = 0;
+    // chained stochastic rounding: the counter of copy `ctr_copy` plus `ctr_add` is this
+    // launch's step number, and the launch leaves the counters alone (ctr_copy < 0: its own)
+    int ctr_copy = -1;
+    unsigned ctr_add = 0;
 };
 
 cudaError_t launch_step_fp32(const StepLaunch& k, const DevParams& p, const void* src, void* dst, cudaStream_t s);

@@ -401,8 +401,9 @@ __global__ void __launch_bounds__(512, 1) tclbm_resident(const __grid_constant__
     }
 }
 
-// Advances the stochastic-rounding counter of a lattice by n steps (after a resident run).
-static __global__ void tclbm_resident_count(const DevParams p, int to, unsigned n) {
+// Advances the stochastic-rounding counter of a lattice by n steps (after a resident run or
+// a chain of launches that left it alone).
+static __global__ void tclbm_count_steps(const DevParams p, int to, unsigned n) {
     p.step_ctr[to] = p.step_ctr[p.parity] + n;
 }
 

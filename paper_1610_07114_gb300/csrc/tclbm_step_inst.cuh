@@ -111,7 +111,9 @@ static long long plain_resident() {
 template <int TX>
 static cudaError_t launch_tx(const StepLaunch& k, const DevParams& p0, const void* src, void* dst, cudaStream_t s) {
     DevParams p = p0;
-    p.parity = k.parity;
+    p.parity = k.ctr_copy < 0 ? k.parity : k.ctr_copy;  // (the kernels index nothing but the counters with it)
+    p.ctr_add = k.ctr_add;
+    p.ctr_hold = k.ctr_copy >= 0;
     const dim3 grid = step_grid(p, TX, k.ty);
     const ST* in = static_cast<const ST*>(src);
     ST* out = static_cast<ST*>(dst);
@@ -257,7 +259,7 @@ static cudaError_t launch_resident_kind(const ResLaunch& r, const DevParams& p0,
     e = cudaLaunchKernelEx(&cfg, kernel, p, static_cast<const ST*>(src), static_cast<ST*>(dst),
                            static_cast<uint4*>(r.board), r.plan.gx, r.plan.gy, r.n, r.tag0, r.err);
     if (e == cudaSuccess && p.rounding) {
-        tclbm_resident_count<<<1, 1, 0, s>>>(p, r.parity ^ 1, (unsigned)r.n);
+        tclbm_count_steps<<<1, 1, 0, s>>>(p, r.parity ^ 1, (unsigned)r.n);
         e = cudaGetLastError();
     }
     return e;
