@@ -508,6 +508,20 @@ __global__ void snapshot_kernel(const DevParams p, const ST* __restrict__ src, f
     }
 }
 
+// Makes the pages of a host output array present, all of which the caller is about to have
+// overwritten.  A device-to-host copy into pages nobody has touched yet (a fresh array of
+// more than a few hundred kilobytes) faults them in one by one from the copy's side: 1.6 to
+// 3 GB/s where touched pages take 120.  The host's own faults cost a tenth of that, and run
+// while the device still works.
+void touch_pages(void* array, size_t bytes) {
+    constexpr size_t kPage = 4096;
+    if (!array || bytes < kPage) return;
+    char* const first = static_cast<char*>(array);
+    const uintptr_t head = reinterpret_cast<uintptr_t>(first) % kPage;
+    *const_cast<volatile char*>(first) = 0;
+    for (size_t i = kPage - head; i < bytes; i += kPage) const_cast<volatile char*>(first)[i] = 0;
+}
+
 int grid_for(long long n, int block) {
     long long g = (n + block - 1) / block;
     if (g > 152 * 16) g = 152 * 16;
@@ -1036,6 +1050,8 @@ tclbm_status tclbm_moments(tclbm_lattice* L, double* rho, double* ux, double* uy
     if (st != TCLBM_OK) return st;
     CK(cudaGetLastError());
     if (!on_device)
+        for (int k = 0; k < 4; ++k) touch_pages(out[k], n * sizeof(double));
+    if (!on_device)
         for (int k = 0; k < 4; ++k)
             if (out[k])
                 CK(cudaMemcpyAsync(out[k], dst[k], n * sizeof(double), cudaMemcpyDeviceToHost, L->stream));
@@ -1113,6 +1129,8 @@ tclbm_status tclbm_get_populations(tclbm_lattice* L, double* f, double* h, int32
     });
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess && !on_device) {
+        touch_pages(f, bytes);
+        if (L->prm.thermal) touch_pages(h, bytes);
         e = cudaMemcpyAsync(f, df, bytes, cudaMemcpyDeviceToHost, L->stream);
         if (e == cudaSuccess && h && L->prm.thermal) e = cudaMemcpyAsync(h, dh, bytes, cudaMemcpyDeviceToHost, L->stream);
     }

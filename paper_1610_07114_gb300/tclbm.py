@@ -386,7 +386,7 @@ class Lattice:
         tclbm_step(self.handle, n)
 
     def moments(self):
-        out = [np.zeros((self.ny, self.nx)) for _ in range(4)]
+        out = [np.empty((self.ny, self.nx)) for _ in range(4)]
         tclbm_moments(self.handle, *[_ptr(o) for o in out], 0)
         return dict(zip(("rho", "ux", "uy", "T"), out))
 
@@ -403,8 +403,8 @@ class Lattice:
         tclbm_snapshot_velocity(self.handle)
 
     def populations(self):
-        f = np.zeros((9, self.ny, self.nx))
-        h = np.zeros((9, self.ny, self.nx)) if self.thermal else None
+        f = np.empty((9, self.ny, self.nx))
+        h = np.empty((9, self.ny, self.nx)) if self.thermal else None
         tclbm_get_populations(self.handle, _ptr(f), _ptr(h), 0)
         return f, h
 
