@@ -516,6 +516,12 @@ __global__ void snapshot_kernel(const DevParams p, const ST* __restrict__ src, f
 void touch_pages(void* array, size_t bytes) {
     constexpr size_t kPage = 4096;
     if (!array || bytes < kPage) return;
+    // pageable memory only: what CUDA knows is present, or not for the host to write
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, array) != cudaSuccess || at.type != cudaMemoryTypeUnregistered) {
+        cudaGetLastError();
+        return;
+    }
     char* const first = static_cast<char*>(array);
     const uintptr_t head = reinterpret_cast<uintptr_t>(first) % kPage;
     *const_cast<volatile char*>(first) = 0;
@@ -564,6 +570,16 @@ bool chainable(const tclbm_lattice* L) {
     return L->kernel == KERNEL_TMA && L->prm.thermal && L->prm.correction && L->ty >= 8 && (tail == 0 || tail >= 3);
 }
 
+// Whether a caller is capturing `s` (a replayed launch would reuse tickets and step numbers).
+bool capturing(cudaStream_t s) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) {
+        cudaGetLastError();
+        return true;
+    }
+    return cap != cudaStreamCaptureStatusNone;
+}
+
 tclbm_status launch_steps(tclbm_lattice* L, int64_t n) {
     if (n > 0 && L->kernel == KERNEL_TMA) {
         tclbm_status st = ensure_maps(L);
@@ -572,7 +588,7 @@ tclbm_status launch_steps(tclbm_lattice* L, int64_t n) {
     // TMA launches with the correction term publish per-item completion tickets; after the
     // first launch of this run the next one waits for each item's neighbours only
     const bool tickets = L->kernel == KERNEL_TMA && L->prm.thermal && L->prm.correction;
-    const bool chain = n > 1 && chainable(L);
+    const bool chain = n > 1 && chainable(L) && !capturing(L->stream);
     const int first = L->cur;
     for (int64_t s = 0; s < n; ++s) {
         StepLaunch k = step_launch(L, L->cur);
@@ -629,12 +645,7 @@ bool resident_planned(tclbm_lattice* L) {
 tclbm_status resident_steps(tclbm_lattice* L, int64_t n, int64_t& done) {
     done = 0;
     if (n < kResMinSteps || !resident_planned(L)) return TCLBM_OK;
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(L->stream, &cap) != cudaSuccess) {
-        cudaGetLastError();
-        return TCLBM_OK;
-    }
-    if (cap != cudaStreamCaptureStatusNone) return TCLBM_OK;
+    if (capturing(L->stream)) return TCLBM_OK;
     if (!L->board) {
         L->board_bytes = 2 * (size_t)L->prm.nx * L->prm.ny * (size_t)(L->nplanes / 3) * 16;
         L->board = dev_alloc(L, L->board_bytes);

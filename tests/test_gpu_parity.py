@@ -661,3 +661,63 @@ def test_resident_runs_equal_one_launch_per_step(T, name, make, storage, roundin
     (fa, ha), (fb, hb) = states
     assert np.array_equal(fa, fb)
     assert not case["thermal"] or np.array_equal(ha, hb)
+
+
+@pytest.mark.parametrize("name,make", [
+    # 16-bit storage with stochastic rounding: the draws' step numbers along a chain
+    ("rb_2048x1024_fp16_sr", lambda: W.rayleigh_benard(2048, 1024, seed=5, storage="fp16")),
+    ("periodic_1536x1409_bf16_sr", lambda: W.random_periodic(1536, 1409, seed=6, force="none", storage="bf16")),
+    # a last strip of three columns, the narrowest that chains
+    ("periodic_1411x800", lambda: W.random_periodic(1411, 800, seed=7, force="accel")),
+    ("xwalls_1027x1100", lambda: W.with_walls(*W.random_periodic(1027, 1100, seed=8, force="accel"), axis="x",
+                                              kind="zouhe")),
+], ids=["rb_2048x1024_fp16_sr", "periodic_1536x1409_bf16_sr", "periodic_1411x800", "xwalls_1027x1100"])
+def test_default_chained_launches_equal_one_step_per_call(T, name, make):
+    # the shape the library picks from 2^20 nodes: 70 steps by one call, against single calls,
+    # which wait for the whole previous grid: bit for bit
+    case, fields = make()
+    case = dict(case, rounding="stochastic" if case.get("storage", "fp32") != "fp32" else "nearest")
+    states = []
+    for calls in ([70], [1] * 70, [1, 3, 1, 65]):
+        lat = T.Lattice(case, fields)
+        assert lat.describe().startswith("tclbm_step_tma_corr"), lat.describe()
+        for n in calls:
+            lat.step(n)
+        states.append(lat.populations())
+        lat.close()
+    for f, h in states[1:]:
+        assert np.array_equal(f, states[0][0]) and np.array_equal(h, states[0][1])
+
+
+@pytest.mark.parametrize("name,make", [
+    ("chained", lambda: W.rayleigh_benard(1536, 768, seed=11)),
+    ("chained_sr", lambda: W.rayleigh_benard(1536, 768, seed=12, storage="fp16")),
+    ("resident", lambda: W.rayleigh_benard(128, 64, seed=13)),
+    ("tiles_sr", lambda: W.rayleigh_benard(512, 256, seed=14, storage="fp16")),
+], ids=["chained", "chained_sr", "resident", "tiles_sr"])
+def test_steps_captured_by_the_caller_replay_like_calls(T, name, make):
+    # ten steps captured in the caller's graph and replayed: every launch then waits for the
+    # whole grid before it, whatever the same call does outside a capture
+    import torch
+
+    case, fields = make()
+    case = dict(case, rounding="stochastic" if case.get("storage", "fp32") != "fp32" else "nearest")
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        lat = T.Lattice(case, fields)
+        lat.step(10)
+    stream.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream, capture_error_mode="thread_local"):
+        lat.step(10)
+    for _ in range(6):
+        with torch.cuda.stream(stream):
+            graph.replay()
+    stream.synchronize()
+    got = lat.populations()
+    lat.close()
+    lat = T.Lattice(case, fields)
+    lat.step(70)
+    exp = lat.populations()
+    lat.close()
+    assert np.array_equal(got[0], exp[0]) and np.array_equal(got[1], exp[1])
