@@ -141,11 +141,11 @@ tclbm_status tclbm_init_fields(tclbm_lattice* lat, const double* rho, const doub
                                const double* T, int32_t on_device);
 
 /* Advance `nsteps` >= 0 time steps (asynchronous on the handle's stream).  Under kernel
- * variant 0 with the correction term (and round-to-nearest for 16-bit storage, rows per
- * CTA >= 8), the launches of one call are chained: each work item of a launch waits
- * only for the nine items around it in the previous launch, so consecutive steps
- * overlap on the device; the first launch of a call waits for whatever precedes it on
- * the stream.  The states are bit-identical to one step per call.  A chained wait that
+ * variant 0 with the correction term (rows per CTA >= 8, a last strip of 3 or more
+ * columns, a stream that is not capturing), the launches of one call are chained: each
+ * work item of a launch waits only for the nine items around it in the previous launch,
+ * so consecutive steps overlap on the device; the first launch of a call waits for
+ * whatever precedes it on the stream.  The states are bit-identical to one step per call.  A chained wait that
  * expires is reported like the other bounded waits (TCLBM_ETIMEOUT at the next
  * synchronising call).
  *
@@ -257,8 +257,9 @@ tclbm_status tclbm_set_tile(tclbm_lattice* lat, int32_t tx, int32_t ty);
  * accelerator, 1 = direct loads marching up strips of rows, 2 = direct loads on 2-D
  * tiles, one node per thread (thermal lattices with the correction term; on a walled x
  * axis nx % BX != 1 and on a walled y axis ny % BY != 1, else TCLBM_EUNSUPPORTED).  The
- * library picks per lattice size: 2 (or 1 where 2 does not apply) up to 2,097,152
- * nodes, 0 above.  Interior nodes evolve bit-identically under all variants; wall
+ * library picks per lattice size: 0 above 2,097,152 nodes, and from 1,048,576 for thermal
+ * lattices with the correction term, 512 or more columns, no work term and launches that
+ * chain; else 2 (or 1 where 2 does not apply).  Interior nodes evolve bit-identically under all variants; wall
  * nodes may differ in the last bit (multiply-add contraction).  Changing the variant
  * resets the launch shape to that variant's default.  EINVAL for other values. */
 tclbm_status tclbm_set_kernel(tclbm_lattice* lat, int32_t kind);
@@ -266,7 +267,8 @@ tclbm_status tclbm_set_kernel(tclbm_lattice* lat, int32_t kind);
 /* ------------------------------------------------------------------ batches
  * A batch advances many independent lattices together: one launch of the batched step
  * kernel per time step over a work list of strips of every lattice (tx columns by
- * `rows` rows each, largest lattices first), captured in CUDA graphs for long runs.
+ * `rows` rows each, largest lattices first; one launch per kernel group, and the groups
+ * run their chains of steps side by side), captured in CUDA graphs for long runs.
  * The paper treats one lattice at a time; a batch changes no arithmetic: every node
  * is updated by the same code as in tclbm_step(), so each lattice evolves exactly as
  * it does alone with the direct-load kernel (tclbm_set_kernel(lat, 1)).

@@ -182,8 +182,9 @@ void derive(tclbm_lattice* L) {
 
 // Lattices that fit in L2 are latency-bound: 2-D tiles of one node per thread (or the
 // direct-load kernel with short strips where tiles do not apply) expose the most
-// parallelism.  Larger lattices stream rows through the TMA ring with 128-wide strips
-// of 16 or 32 rows per CTA (default_shape).
+// parallelism (runs of 8 or more steps of lattices that fit in shared memory stay there:
+// resident_steps).  Larger lattices stream rows through the TMA ring in 128-wide strips
+// (rows per CTA: default_shape).
 constexpr long long kSmallNodes = 1LL << 21, kChainNodes = 1LL << 20;
 
 // Launch shape a kernel variant gets by default: (tx, rows per CTA) for the marching
