@@ -384,6 +384,16 @@ struct CorrShape {
     static constexpr int kThreadsPerSM = sizeof(ST) == 4 ? 384 : 512;
 };
 
+// The same for the batched kernel.  Its constants are shared-memory loads, and at four CTAs
+// of 128 threads the 16-bit strips spill 216 to 244 bytes a thread.  64-wide strips run six
+// CTAs without them: 48 lattices of 64 x 32 to 1024 x 512 in FP16, 32 rows, 257 -> 230 us a
+// step (16 rows 264 -> 244); 128-wide strips gain nothing at three (32 rows 224 / 223, 16
+// rows 229 / 233).
+template <int TX, class ST>
+struct BatchCorrShape {
+    static constexpr int kThreadsPerSM = TX == 64 ? 384 : CorrShape<ST>::kThreadsPerSM;
+};
+
 // One strip: columns [x0, x0 + TX) of rows [y0, y1), every thread of the CTA.  `p` is a
 // kernel parameter or a shared-memory copy; `map` the source copy's tensor map (in
 // parameter or global memory); `smem` the dynamic shared memory of tma_smem_bytes().
@@ -648,7 +658,7 @@ __global__ void __launch_bounds__(TX, CorrShape<ST>::kThreadsPerSM / TX) tclbm_s
 // does alone with that kernel.  A lattice whose error word is set is skipped; an
 // expired wait sets it.
 template <int TX, class ST>
-__global__ void __launch_bounds__(TX, CorrShape<ST>::kThreadsPerSM / TX) tclbm_step_batch_tma(
+__global__ void __launch_bounds__(TX, BatchCorrShape<TX, ST>::kThreadsPerSM / TX) tclbm_step_batch_tma(
     const BatchLattice* __restrict__ lats, const BatchItem* __restrict__ items, int nitems, int step_parity) {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ DevParams sp;
