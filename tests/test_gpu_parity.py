@@ -721,3 +721,29 @@ def test_steps_captured_by_the_caller_replay_like_calls(T, name, make):
     exp = lat.populations()
     lat.close()
     assert np.array_equal(got[0], exp[0]) and np.array_equal(got[1], exp[1])
+
+
+@pytest.mark.parametrize("name,make", [
+    ("resident", lambda: W.rayleigh_benard(96, 48, seed=15, storage="fp16")),
+    ("resident_athermal", lambda: _tg(64, storage="bf16")),
+    ("chained", lambda: W.rayleigh_benard(1536, 768, seed=16, storage="fp16")),
+], ids=["resident", "resident_athermal", "chained"])
+def test_draws_after_new_fields_do_not_depend_on_the_launches_before(T, name, make):
+    # stochastic rounding goes on with its step numbers when new fields are set: runs of odd and
+    # even length by one call each against one step per call, bit for bit
+    case, fields = make()
+    case = dict(case, rounding="stochastic")
+    states = []
+    for single in (False, True):
+        lat = T.Lattice(case, fields)
+        got = []
+        for n, again in ((12, True), (11, True), (10, False), (9, True), (1, True), (8, False), (3, True), (13, True)):
+            for k in ([1] * n if single else [n]):
+                lat.step(k)
+            got.append(lat.populations()[0])
+            if again:
+                lat.init_fields(fields)
+        states.append(got)
+        lat.close()
+    for a, b in zip(*states):
+        assert np.array_equal(a, b)
