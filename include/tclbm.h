@@ -244,6 +244,12 @@ tclbm_status tclbm_test_skip_row(tclbm_lattice* lat, int32_t row);
  * EINVAL on n < 0 or NULL arrays with n > 0. */
 tclbm_status tclbm_test_rcp(const float* x, float* y, int64_t n, void* stream);
 
+/* Test hook for the node order of the field conversions (no counterpart in the paper; host
+ * code, no device work): x[k], y[k] = column and row, in a lattice nx wide, of node
+ * first + k * stride as a thread of the conversion kernels counts them, for k < count.
+ * EINVAL on nx < 1, count < 0 or NULL arrays with count > 0. */
+tclbm_status tclbm_test_node_walk(uint32_t first, uint32_t stride, int32_t nx, int64_t count, int32_t* x, int32_t* y);
+
 /* Launch-shape override for tuning; 0 keeps the library's choice.  Kernel variants 0
  * and 1: strip width tx (32, 64 or 128 nodes) and rows per CTA ty (>= 1); under variant 0,
  * where the grid spans more than two waves of resident CTAs, ty is a multiple of 16 and

@@ -273,8 +273,10 @@ __global__ void init_kernel(const DevParams p, const double* __restrict__ rho, c
                             int thermal, double R, double T0, double b, int force_kind, double ax, double ay,
                             double famp) {
     const long long n = (long long)p.nx * p.ny;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const int y = (int)((unsigned)i / (unsigned)p.nx), x = (int)((unsigned)i - (unsigned)y * (unsigned)p.nx);
+    NodeWalk w(blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x, p.nx);
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
+         i += (long long)gridDim.x * blockDim.x, w.next(p.nx)) {
+        const int x = w.x, y = w.y;
         const double r = rho[i], vx = ux[i], vy = uy[i], t = thermal ? T[i] : T0;
         const double RT = __dmul_rn(R, t), ux2 = __dmul_rn(vx, vx), uy2 = __dmul_rn(vy, vy);
         const double qx = __dadd_rn(RT, ux2), qy = __dadd_rn(RT, uy2);
@@ -362,8 +364,10 @@ __global__ void set_pops_kernel(const DevParams p, const double* __restrict__ f,
                                 ST* __restrict__ dst, int thermal) {
     const long long n = (long long)p.nx * p.ny;
     const int ex[9] = {0, 1, 0, -1, 0, 1, -1, -1, 1}, ey[9] = {0, 0, 1, 0, -1, 1, 1, -1, -1};
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const int y = (int)((unsigned)i / (unsigned)p.nx), x = (int)((unsigned)i - (unsigned)y * (unsigned)p.nx);
+    NodeWalk w(blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x, p.nx);
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
+         i += (long long)gridDim.x * blockDim.x, w.next(p.nx)) {
+        const int x = w.x, y = w.y;
 #pragma unroll
         for (int q = 0; q < 9; ++q) {
             int xs = x - ex[q], ys = y - ey[q];
@@ -381,8 +385,10 @@ template <bool THERMAL, class ST>
 __global__ void get_pops_kernel(const DevParams p, const ST* __restrict__ src, double* __restrict__ f,
                                 double* __restrict__ h) {
     const long long n = (long long)p.nx * p.ny;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const int y = (int)((unsigned)i / (unsigned)p.nx), x = (int)((unsigned)i - (unsigned)y * (unsigned)p.nx);
+    NodeWalk w(blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x, p.nx);
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
+         i += (long long)gridDim.x * blockDim.x, w.next(p.nx)) {
+        const int x = w.x, y = w.y;
         float fv[9], hv[9];
         load_node<THERMAL, ST>(p, src, x, y, fv, hv);
 #pragma unroll
@@ -398,8 +404,10 @@ template <bool THERMAL, class ST>
 __global__ void moments_kernel(const DevParams p, const ST* __restrict__ src, double* __restrict__ rho,
                                double* __restrict__ ux, double* __restrict__ uy, double* __restrict__ T) {
     const long long n = (long long)p.nx * p.ny;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const int y = (int)((unsigned)i / (unsigned)p.nx), x = (int)((unsigned)i - (unsigned)y * (unsigned)p.nx);
+    NodeWalk w(blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x, p.nx);
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
+         i += (long long)gridDim.x * blockDim.x, w.next(p.nx)) {
+        const int x = w.x, y = w.y;
         float fv[9], hv[9];
         load_node<THERMAL, ST>(p, src, x, y, fv, hv);
         const NodeSums s = node_sums<THERMAL>(fv, hv);
@@ -429,8 +437,10 @@ __global__ void __launch_bounds__(kDiagBlock) diag_kernel(const DevParams p, con
     // the linear sums stay FP32 error-free sums of deviations until the thread's last node
     Running drho, jx, jy, sdh;
     double nodes = 0, Fxs = 0, Fys = 0;  // nodes seen, and their Taylor-Green forces
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const int y = (int)((unsigned)i / (unsigned)p.nx), x = (int)((unsigned)i - (unsigned)y * (unsigned)p.nx);
+    NodeWalk w(blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x, p.nx);
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
+         i += (long long)gridDim.x * blockDim.x, w.next(p.nx)) {
+        const int x = w.x, y = w.y;
         float fv[9], hv[9];
         load_node<THERMAL, ST>(p, src, x, y, fv, hv);
         const NodeSums s = node_sums<THERMAL>(fv, hv);
@@ -499,8 +509,10 @@ __global__ void diag_finish(const double* __restrict__ partial, int nblocks, con
 template <bool THERMAL, class ST>
 __global__ void snapshot_kernel(const DevParams p, const ST* __restrict__ src, float* __restrict__ usnap) {
     const long long n = (long long)p.nx * p.ny;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const int y = (int)((unsigned)i / (unsigned)p.nx), x = (int)((unsigned)i - (unsigned)y * (unsigned)p.nx);
+    NodeWalk w(blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x, p.nx);
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
+         i += (long long)gridDim.x * blockDim.x, w.next(p.nx)) {
+        const int x = w.x, y = w.y;
         float fv[9], hv[9];
         load_node<THERMAL, ST>(p, src, x, y, fv, hv);
         const NodeFields v = node_velocity(p, node_sums<false>(fv, hv), x, y);
@@ -951,6 +963,16 @@ tclbm_status tclbm_test_rcp(const float* x, float* y, int64_t n, void* stream) {
     rcp_kernel<<<grid_for(n, 256), 256, 0, s>>>(x, y, n);
     CK(cudaGetLastError());
     CK(cudaStreamSynchronize(s));
+    return TCLBM_OK;
+}
+
+tclbm_status tclbm_test_node_walk(uint32_t first, uint32_t stride, int32_t nx, int64_t count, int32_t* x, int32_t* y) {
+    if (nx < 1 || count < 0 || (count > 0 && (!x || !y))) return fail(TCLBM_EINVAL, "bad node walk");
+    NodeWalk w(first, stride, nx);
+    for (int64_t k = 0; k < count; ++k, w.next(nx)) {
+        x[k] = w.x;
+        y[k] = w.y;
+    }
     return TCLBM_OK;
 }
 

@@ -23,6 +23,27 @@
 
 namespace tclbm {
 
+// Column and row of the nodes first, first + stride, ... that one thread of a conversion
+// visits: two divisions, and an addition with carry from node to node.  `first` and `stride` are
+// numbers of threads (below 2^32); the nodes may go beyond that, where a 32-bit division of the
+// node number would give wrong rows (a lattice has up to 2^34 nodes).
+struct NodeWalk {
+    int x, y, dx, dy;
+    __host__ __device__ __forceinline__ NodeWalk(unsigned first, unsigned stride, int nx) {
+        const unsigned m = (unsigned)nx, fy = first / m, sy = stride / m;
+        y = (int)fy;
+        x = (int)(first - fy * m);
+        dy = (int)sy;
+        dx = (int)(stride - sy * m);
+    }
+    __host__ __device__ __forceinline__ void next(int nx) {
+        const unsigned t = (unsigned)x + (unsigned)dx;  // (below 2 nx < 2^32)
+        const bool over = t >= (unsigned)nx;
+        x = (int)(over ? t - (unsigned)nx : t);
+        y += dy + (over ? 1 : 0);
+    }
+};
+
 // (double)v without the FP64 pipe for zeros and normal numbers.
 __device__ __forceinline__ double f2d(float v) {
     const unsigned u = __float_as_uint(v), m = u & 0x7fffffffu;

@@ -100,6 +100,9 @@ _lib.tclbm_test_skip_row.argtypes = [_vp, ctypes.c_int32]
 _lib.tclbm_test_skip_row.restype = ctypes.c_int
 _lib.tclbm_test_rcp.argtypes = [_vp, _vp, ctypes.c_int64, _vp]
 _lib.tclbm_test_rcp.restype = ctypes.c_int
+_i32p = ctypes.POINTER(ctypes.c_int32)
+_lib.tclbm_test_node_walk.argtypes = [ctypes.c_uint32, ctypes.c_uint32, ctypes.c_int32, ctypes.c_int64, _i32p, _i32p]
+_lib.tclbm_test_node_walk.restype = ctypes.c_int
 _lib.tclbm_set_kernel.argtypes = [_vp, ctypes.c_int32]
 _lib.tclbm_set_kernel.restype = ctypes.c_int
 _lib.tclbm_copy_rows.argtypes = [_vp, ctypes.c_int32, _vp, ctypes.c_int32, ctypes.c_int32]
@@ -210,6 +213,13 @@ def tclbm_test_skip_row(h, row):
 
 def tclbm_test_rcp(x, y, n, stream=None):
     _check(_lib.tclbm_test_rcp(x, y, int(n), stream), "tclbm_test_rcp")
+
+
+def tclbm_test_node_walk(first, stride, nx, count):
+    x, y = np.zeros(count, dtype=np.int32), np.zeros(count, dtype=np.int32)
+    _check(_lib.tclbm_test_node_walk(first, stride, nx, count, x.ctypes.data_as(_i32p), y.ctypes.data_as(_i32p)),
+           "tclbm_test_node_walk")
+    return x, y
 
 
 def tclbm_copy_rows(dst, dst_row, src, src_row, rows):

@@ -81,3 +81,16 @@ def test_zero_flux_adiabatic_walls_are_refused_by_the_cuda_path(T):
     T.params_from_case(case)
     with pytest.raises(ValueError):
         T.params_from_case(dict(case, adiabatic="zero_flux"))
+
+
+@pytest.mark.parametrize("nx", [1, 3, 511, 65536, 92683, (1 << 20) + 7, (1 << 31) - 1])
+@pytest.mark.parametrize("first,stride", [(0, 1 << 31), (77, 622592 * 997), ((1 << 32) - 1, (1 << 32) - 1)])
+def test_nodes_beyond_32_bits_keep_their_rows(T, nx, first, stride):
+    # the conversion kernels find a node's place from its 64-bit number: strides that carry the
+    # count past 2^32 (the largest lattice has 2^34 nodes), against 64-bit arithmetic
+    count = 9 if nx > 3 else 2  # (rows stay below 2^31)
+    x, y = T.tclbm_test_node_walk(first, stride, nx, count)
+    for k in range(count):
+        node = first + k * stride
+        if node // nx < 1 << 31:
+            assert (int(x[k]), int(y[k])) == (node % nx, node // nx), (node, nx)
