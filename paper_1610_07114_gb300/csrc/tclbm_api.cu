@@ -692,7 +692,8 @@ tclbm_status resident_steps(tclbm_lattice* L, int64_t n, int64_t& done) {
         r.tag0 = L->res_tag;
         r.board = L->board;
         r.err = L->err;
-        const cudaError_t e = launch_resident(L->prm.storage, r, L->dp, L->buf[L->cur], L->buf[L->cur ^ 1], L->stream);
+        const int to = L->cur ^ (int)(k & 1);  // the copy that k launches would end in
+        const cudaError_t e = launch_resident(L->prm.storage, r, L->dp, L->buf[L->cur], L->buf[to], L->stream);
         if (e == cudaErrorCooperativeLaunchTooLarge) {  // fewer multiprocessors than the device has are ours
             cudaGetLastError();
             L->res_state = -1;
@@ -700,7 +701,7 @@ tclbm_status resident_steps(tclbm_lattice* L, int64_t n, int64_t& done) {
         }
         if (e != cudaSuccess) return cuda_fail(e, "resident kernel launch");
         L->res_tag += (unsigned)k;
-        L->cur ^= 1;
+        L->cur = to;
         L->steps += k;
         done += k;
     }

@@ -87,7 +87,8 @@ cudaError_t prepare_step_fp32();
 cudaError_t prepare_step_bf16();
 cudaError_t prepare_step_fp16();
 
-// Resident run of n steps (tclbm_resident.cuh) from `src` to `dst` under `plan`.
+// Resident run of n steps (tclbm_resident.cuh) from `src` to `dst` (n even: the same copy)
+// under `plan`.
 struct ResLaunch {
     ResPlan plan;
     int kind;  // RES_*

@@ -19,6 +19,12 @@
 // numbers only grow over the life of a lattice, so what an earlier launch left on the
 // board never matches.
 //
+// A run of an even number of steps ends in the copy it started from, as that many launches
+// would (work that a caller captured earlier reads that copy).  Updating in place is safe:
+// only a tile and the tiles around it read its nodes from the source copy, all before the
+// first publication, and a CTA stores its last state after it has read publications of every
+// tile around it.
+//
 // What bounds it: the exchange (a store through L2 to a neighbour's read, 1 to 1.5 us) and
 // the dependent chain of one node update (about 1 us at one or two warps per scheduler).
 // Measured (GB300, us per step against one launch per step): thermal with the correction
@@ -135,11 +141,11 @@ struct ResNode {
     int one_x, one_y;  // one-sided derivative: +1 at the lower wall, -1 at the upper, 0 none
 };
 
-// n steps of the lattice from `src` to `dst`.  MULTI: more nodes than threads; a node is
+// n >= 2 steps of the lattice from `src` to `dst`, which may be the same copy.  MULTI: more nodes than threads; a node is
 // then pulled once for its moments and again for its collision.
 template <class ST, int KIND, bool MULTI, bool FAST>
-__global__ void __launch_bounds__(512, 1) tclbm_resident(const __grid_constant__ DevParams p, const ST* __restrict__ src,
-                                                         ST* __restrict__ dst, uint4* __restrict__ board, int gx, int gy,
+__global__ void __launch_bounds__(512, 1) tclbm_resident(const __grid_constant__ DevParams p, const ST* src,
+                                                         ST* dst, uint4* __restrict__ board, int gx, int gy,
                                                          int n, unsigned tag0, int* __restrict__ err) {
     using S = ResShape<KIND, MULTI>;
     constexpr int R = S::R, NP = S::NP, CELLS = S::CELLS, W = S::W, ITEMS = 4;
@@ -172,7 +178,8 @@ __global__ void __launch_bounds__(512, 1) tclbm_resident(const __grid_constant__
         if (p.yper) y = ((y % ny) + ny) % ny; else valid = valid && y >= 0 && y < ny;
 #pragma unroll
         for (int q = 0; q < NP; ++q)
-            frame[q * CELLS + c] = valid ? Store<ST>::ld(src + q * p.plane + ((long long)y * p.pitch + x)) : 0.0f;
+            // (an ordinary load, not the read-only path: dst may be src)
+            frame[q * CELLS + c] = valid ? Store<ST>::ld_smem(src + q * p.plane + ((long long)y * p.pitch + x)) : 0.0f;
         if (!valid)  // past a wall: never written again, and replaced by the wall scheme where it is pulled
 #pragma unroll
             for (int q = 0; q < NP; ++q) frame[(NP + q) * CELLS + c] = 0.0f;

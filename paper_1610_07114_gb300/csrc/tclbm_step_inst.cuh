@@ -259,7 +259,7 @@ static cudaError_t launch_resident_kind(const ResLaunch& r, const DevParams& p0,
     e = cudaLaunchKernelEx(&cfg, kernel, p, static_cast<const ST*>(src), static_cast<ST*>(dst),
                            static_cast<uint4*>(r.board), r.plan.gx, r.plan.gy, r.n, r.tag0, r.err);
     if (e == cudaSuccess && p.rounding) {
-        tclbm_count_steps<<<1, 1, 0, s>>>(p, r.parity ^ 1, (unsigned)r.n);
+        tclbm_count_steps<<<1, 1, 0, s>>>(p, r.parity ^ (r.n & 1), (unsigned)r.n);
         e = cudaGetLastError();
     }
     return e;

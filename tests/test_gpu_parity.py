@@ -747,3 +747,39 @@ def test_draws_after_new_fields_do_not_depend_on_the_launches_before(T, name, ma
         lat.close()
     for a, b in zip(*states):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("name,make", [
+    ("fp32", lambda: W.rayleigh_benard(128, 64, seed=18)),
+    ("fp16_sr", lambda: W.rayleigh_benard(96, 48, seed=19, storage="fp16")),
+    ("athermal", lambda: _tg(64, storage="bf16")),
+    ("one_tile", lambda: W.random_periodic(9, 7, seed=20)),
+], ids=["fp32", "fp16_sr", "athermal", "one_tile"])
+def test_captured_steps_replay_after_runs_of_an_even_length(T, name, make):
+    # six steps captured by the caller, replayed between calls of 10, 2 and 4104 steps: the
+    # state has to be where the capture reads it after any even number of steps
+    import torch
+
+    case, fields = make()
+    case = dict(case, rounding="stochastic" if case.get("storage", "fp32") != "fp32" else "nearest")
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        lat = T.Lattice(case, fields)
+    stream.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream, capture_error_mode="thread_local"):
+        lat.step(6)
+    for n in (10, 2, 4104):
+        with torch.cuda.stream(stream):
+            lat.step(n)
+            graph.replay()
+    stream.synchronize()
+    got = lat.populations()
+    lat.close()
+    lat = T.Lattice(case, fields)
+    lat.set_kernel(2 if lat.describe().startswith("tclbm_step_tile") else 1)
+    lat.step(10 + 2 + 4104 + 3 * 6)
+    exp = lat.populations()
+    lat.close()
+    assert np.array_equal(got[0], exp[0])
+    assert not case["thermal"] or np.array_equal(got[1], exp[1])
