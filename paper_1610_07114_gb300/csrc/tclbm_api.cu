@@ -1045,15 +1045,7 @@ tclbm_status tclbm_init_fields(tclbm_lattice* L, const double* rho, const double
     });
     if (st != TCLBM_OK) return st;
     CK(cudaGetLastError());
-    if (L->dp.rounding && (L->cur != 0 || (L->steps & 1))) {
-        // The draws go on from the count that copy 0 of the counter holds.  One launch per step
-        // leaves all steps there after an even number, one fewer after an odd one; a chained or
-        // resident run of the same steps has to leave the same.
-        DevParams q = L->dp;
-        q.parity = L->cur;
-        tclbm_count_steps<<<1, 1, 0, L->stream>>>(q, 0, (unsigned)-(int)(L->steps & 1));
-        CK(cudaGetLastError());
-    }
+    // (the draws go on from copy 0 of the step counter: tclbm_count_steps)
     L->cur = 0;
     L->steps = 0;
     if (!on_device) CK(cudaStreamSynchronize(L->stream));  // host arrays may be freed on return

@@ -408,10 +408,15 @@ __global__ void __launch_bounds__(512, 1) tclbm_resident(const __grid_constant__
     }
 }
 
-// Advances the stochastic-rounding counter of a lattice by n steps (after a resident run or
-// a chain of launches that left it alone).
+// Advances the stochastic-rounding counters of a lattice by n >= 1 steps (after a resident run
+// or a chain of launches that left them alone): `to` is the copy the state ended in.  Both get
+// what one launch per step would leave in them -- all steps in the copy of the state, one
+// fewer in the other -- so that new fields, which always start from copy 0, and launches that a
+// caller captured earlier go on with the same draws whatever ran before.
 static __global__ void tclbm_count_steps(const DevParams p, int to, unsigned n) {
-    p.step_ctr[to] = p.step_ctr[p.parity] + n;
+    const unsigned total = p.step_ctr[p.parity] + n;
+    p.step_ctr[to] = total;
+    p.step_ctr[to ^ 1] = total - 1u;
 }
 
 }  // namespace tclbm

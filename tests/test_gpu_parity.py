@@ -783,3 +783,38 @@ def test_captured_steps_replay_after_runs_of_an_even_length(T, name, make):
     lat.close()
     assert np.array_equal(got[0], exp[0])
     assert not case["thermal"] or np.array_equal(got[1], exp[1])
+
+
+def test_new_fields_in_a_captured_graph_continue_the_draws(T):
+    # new fields and four steps captured while the state is in copy 1, replayed three times:
+    # the draws go on from replay to replay as they do call by call, bit for bit
+    import torch
+
+    case, fields = W.rayleigh_benard(96, 48, seed=17, storage="fp16")
+    case = dict(case, rounding="stochastic")
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        lat = T.Lattice(case, fields)
+        dev = {k: torch.as_tensor(v, dtype=torch.float64, device="cuda") for k, v in fields.items()}
+        lat.step(11)
+    stream.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream, capture_error_mode="thread_local"):
+        lat.init_fields(dev)
+        lat.step(4)
+    for _ in range(3):
+        with torch.cuda.stream(stream):
+            graph.replay()
+    stream.synchronize()
+    got = lat.populations()
+    lat.close()
+    lat = T.Lattice(case, fields)
+    for _ in range(11):
+        lat.step(1)
+    for _ in range(3):
+        lat.init_fields(fields)
+        for _ in range(4):
+            lat.step(1)
+    exp = lat.populations()
+    lat.close()
+    assert np.array_equal(got[0], exp[0]) and np.array_equal(got[1], exp[1])
