@@ -507,8 +507,8 @@ def bench_gpu(args):
         "serving": serving,
         "cpu_baseline": cpu,
         "clocks": clk,
-        # (a resident run takes up to 4096 steps in one launch)
-        "gpu_launches": args.steps * ((-(-args.chunk // 4096) if "tclbm_resident" in desc else args.chunk) + 2),
+        # (a resident run takes up to 1024 steps in one launch)
+        "gpu_launches": args.steps * ((-(-args.chunk // 1024) if "tclbm_resident" in desc else args.chunk) + 2),
         "nusselt": nu_num,
         "kernel_us": kernel_s * 1e6,
     }

@@ -152,8 +152,11 @@ tclbm_status tclbm_init_fields(tclbm_lattice* lat, const double* rho, const doub
  * A lattice small enough for the shared memory of the device (about 60,000 nodes with the
  * correction term, 190,000 without, 390,000 athermal; no work term) whose kernel and
  * launch shape are the library's choice takes 8 or more steps in cooperative launches that
- * keep its state resident (up to 4096 steps each), unless the stream is capturing.  The
- * states are the same bit for bit.  The first such call allocates, through the hooks, an
+ * keep its state resident (up to 1024 steps each), unless the stream is capturing.  Such a
+ * launch keeps the multiprocessors it uses to itself, so where handles of this process are on
+ * more than one stream of the device only lattices that fit on it eight times over (2000
+ * nodes or so with the correction term, 6000 athermal) run resident; the others then take one
+ * launch per step, which share the device.  The states are the same bit for bit.  The first such call allocates, through the hooks, an
  * exchange board of 192 bytes per node (96 athermal); without it the lattice takes one
  * launch per step.  The bounded waits of these launches are reported in the same way. */
 tclbm_status tclbm_step(tclbm_lattice* lat, int64_t nsteps);

@@ -15,6 +15,7 @@
 #include <cstdio>
 #include <cstdarg>
 #include <cstring>
+#include <mutex>
 #include <type_traits>
 #include <new>
 
@@ -48,6 +49,55 @@ constexpr int kDiagMaxBlocks = 1024;
 }  // namespace
 
 void tclbm::set_last_error(const char* msg) { snprintf(g_err, sizeof g_err, "%s", msg); }
+
+struct tclbm::StreamUse {
+    int dev;
+    cudaStream_t stream;
+    int handles;
+    StreamUse* next;
+};
+
+namespace {
+std::mutex g_use_mutex;
+StreamUse* g_uses = nullptr;
+}  // namespace
+
+StreamUse* tclbm::use_stream(cudaStream_t s) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    std::lock_guard<std::mutex> lock(g_use_mutex);
+    // (the per-thread stream is another one in each thread: an entry for each handle)
+    if (s != cudaStreamPerThread)
+        for (StreamUse* u = g_uses; u; u = u->next)
+            if (u->dev == dev && u->stream == s) {
+                ++u->handles;
+                return u;
+            }
+    StreamUse* u = new (std::nothrow) StreamUse{dev, s, 1, g_uses};
+    if (u) g_uses = u;
+    return u;
+}
+
+void tclbm::unuse_stream(StreamUse* u) {
+    if (!u) return;
+    std::lock_guard<std::mutex> lock(g_use_mutex);
+    if (--u->handles > 0) return;
+    StreamUse** at = &g_uses;
+    while (*at != u) at = &(*at)->next;
+    *at = u->next;
+    delete u;
+}
+
+bool tclbm::only_stream(const StreamUse* u) {
+    if (!u) return false;
+    std::lock_guard<std::mutex> lock(g_use_mutex);
+    for (const StreamUse* v = g_uses; v; v = v->next)
+        if (v != u && v->dev == u->dev) return false;
+    return true;
+}
 
 void* tclbm::dev_alloc(tclbm_lattice* L, size_t bytes) {
     if (bytes == 0) return nullptr;
@@ -640,13 +690,24 @@ tclbm_status launch_steps(tclbm_lattice* L, int64_t n) {
     return TCLBM_OK;
 }
 
-// Steps of one resident launch at most (a few milliseconds), and the fewest steps worth one:
-// filling and emptying the shared memory costs about as much as two steps.
-constexpr int64_t kResMaxSteps = 4096, kResMinSteps = 8;
+// Steps of one resident launch at most (1.5 to 6 ms, which work of other streams may have to
+// wait for), and the fewest steps worth one: filling and emptying the shared memory costs
+// about as much as two steps.
+constexpr int64_t kResMaxSteps = 1024, kResMinSteps = 8;
+
+// Resident launches of one lattice that the device has to hold at once for lattices on several
+// streams to run so.  A resident launch keeps its multiprocessors to itself for hundreds of
+// steps, where one-step launches of several lattices share them.  Measured (us per step of all,
+// K lattices on streams of their own, resident / one launch per step): 64 x 32 thermal with the
+// correction term (15 fit) K = 4 2.6 / 3.1, K = 16 3.7 / 6.5; 64 x 64 (7.6 fit) K = 8 4.0 / 3.5;
+// 256 x 128 (1 fits) K = 2 5.9 / 4.0, K = 16 47.7 / 18.7; athermal 80 x 80 (9.5 fit) K = 16
+// 3.6 / 8.8, 192 x 192 (2.0 fit) K = 8 8.5 / 5.4.
+constexpr long long kResShared = 8;
 
 int res_kind(const tclbm_params& p) { return !p.thermal ? RES_ATHERMAL : (p.correction ? RES_CORR : RES_THERMAL); }
 
-// Whether L runs resident where enough steps are asked for (planned on first use).
+// Whether L runs resident where enough steps are asked for (planned on first use): the library
+// chose its kernel and shape, it fits, and it has the device to itself or takes little of it.
 bool resident_planned(tclbm_lattice* L) {
     if (!L->auto_kernel || L->dp.work) return false;
     if (L->res_state == 0) {
@@ -657,8 +718,11 @@ bool resident_planned(tclbm_lattice* L) {
             coop = 0;
         }
         L->res_state = coop && res_plan(L->dp, res_kind(L->prm), sm_count(), L->res_plan) ? 1 : -1;
+        if (L->res_state > 0)
+            L->res_small = (long long)resident_per_sm(L->storage, res_kind(L->prm), L->res_plan, L->dp) * sm_count() >=
+                           kResShared * L->res_plan.gx * L->res_plan.gy;
     }
-    return L->res_state > 0;
+    return L->res_state > 0 && (L->res_small || only_stream(L->use));
 }
 
 // Advances L by as many of n steps as resident launches take (`done`); 0 where they do not
@@ -900,6 +964,7 @@ tclbm_status tclbm_create(const tclbm_params* params, tclbm_alloc_fn alloc, tclb
         }
     }
     snprintf(L->desc, sizeof L->desc, "unset");
+    L->use = use_stream(L->stream);
     *out = L;
     return TCLBM_OK;
 }
@@ -918,13 +983,17 @@ tclbm_status tclbm_destroy(tclbm_lattice* L) {
     dev_free(L, L->seg_done, L->seg_bytes);
     dev_free(L, L->board, L->board_bytes);
     if (L->copy_event) cudaEventDestroy(L->copy_event);
+    unuse_stream(L->use);
     delete L;
     return TCLBM_OK;
 }
 
 tclbm_status tclbm_set_stream(tclbm_lattice* L, void* stream) {
     if (!L) return fail(TCLBM_EINVAL, "lattice is NULL");
+    if (L->stream == (cudaStream_t)stream) return TCLBM_OK;
+    unuse_stream(L->use);
     L->stream = (cudaStream_t)stream;
+    L->use = use_stream(L->stream);
     return TCLBM_OK;
 }
 

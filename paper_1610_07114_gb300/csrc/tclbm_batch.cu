@@ -63,6 +63,7 @@ struct tclbm_batch {
     // the batch stream and join them again (created where a batch has several groups)
     cudaStream_t side[3] = {nullptr, nullptr, nullptr};
     cudaEvent_t fork = nullptr, join[3] = {nullptr, nullptr, nullptr};
+    tclbm::StreamUse* use = nullptr;  // the batch stream among the streams in use
     char desc[256] = "";
 };
 
@@ -419,6 +420,7 @@ tclbm_status tclbm_batch_create(tclbm_lattice* const* lattices, int32_t count, v
         tclbm_batch_destroy(B);
         return st;
     }
+    B->use = use_stream(B->stream);
     *out = B;
     return TCLBM_OK;
 }
@@ -649,6 +651,7 @@ tclbm_status tclbm_batch_destroy(tclbm_batch* B) {
     release(B, p, B->d_items_bytes);
     p = B->d_lats;
     release(B, p, B->d_lats_bytes);
+    unuse_stream(B->use);
     delete B;
     return TCLBM_OK;
 }

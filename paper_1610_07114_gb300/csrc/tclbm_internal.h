@@ -12,6 +12,13 @@
 
 namespace tclbm {
 constexpr int kGraphPairs = 32;  // a captured step graph holds 2 * kGraphPairs launches
+
+// The streams that the handles of this process step on, by device: launches that fill the
+// device shut the work of other streams out, so they are for a device with one such stream.
+struct StreamUse;
+StreamUse* use_stream(cudaStream_t s);  // on the current device; nullptr: not kept track of
+void unuse_stream(StreamUse* u);
+bool only_stream(const StreamUse* u);
 }  // namespace tclbm
 
 using tclbm::DevParams;
@@ -54,6 +61,8 @@ struct tclbm_lattice {
     // number of the last state a run has used
     bool auto_kernel = true;
     int res_state = 0;  // 0 not planned yet, 1 planned, -1 does not apply
+    bool res_small = false;  // several such runs fit on the device at once
+    tclbm::StreamUse* use = nullptr;  // this handle's entry in the streams in use
     tclbm::ResPlan res_plan{};
     void* board = nullptr;
     size_t board_bytes = 0;

@@ -109,6 +109,16 @@ inline cudaError_t launch_resident(int storage, const ResLaunch& r, const DevPar
     }
 }
 
+// CTAs of a plan's kernel that one multiprocessor holds (0: the query failed).
+int resident_per_sm_fp32(int kind, const ResPlan& plan, const DevParams& p);
+int resident_per_sm_bf16(int kind, const ResPlan& plan, const DevParams& p);
+int resident_per_sm_fp16(int kind, const ResPlan& plan, const DevParams& p);
+inline int resident_per_sm(int storage, int kind, const ResPlan& plan, const DevParams& p) {
+    return storage == 0   ? resident_per_sm_fp32(kind, plan, p)
+           : storage == 1 ? resident_per_sm_bf16(kind, plan, p)
+                          : resident_per_sm_fp16(kind, plan, p);
+}
+
 // Tiles of a resident run on `sms` CTAs (false: the lattice does not fit).  A CTA takes at
 // least kResMinNodes nodes: below that a step is all latency and more CTAs only add halo.
 constexpr int kResMinNodes = 96;

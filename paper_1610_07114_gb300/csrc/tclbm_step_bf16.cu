@@ -10,4 +10,5 @@ using ST = __nv_bfloat16;
 #define BATCH_TMA_FN launch_batch_tma_bf16
 #define TMA_RESIDENT_FN tma_resident_bf16
 #define RESIDENT_FN launch_resident_bf16
+#define RESIDENT_OCC_FN resident_per_sm_bf16
 #include "tclbm_step_inst.cuh"

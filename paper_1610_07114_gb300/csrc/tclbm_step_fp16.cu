@@ -10,4 +10,5 @@ using ST = __half;
 #define BATCH_TMA_FN launch_batch_tma_fp16
 #define TMA_RESIDENT_FN tma_resident_fp16
 #define RESIDENT_FN launch_resident_fp16
+#define RESIDENT_OCC_FN resident_per_sm_fp16
 #include "tclbm_step_inst.cuh"

@@ -10,4 +10,5 @@ using ST = float;
 #define BATCH_TMA_FN launch_batch_tma_fp32
 #define TMA_RESIDENT_FN tma_resident_fp32
 #define RESIDENT_FN launch_resident_fp32
+#define RESIDENT_OCC_FN resident_per_sm_fp32
 #include "tclbm_step_inst.cuh"

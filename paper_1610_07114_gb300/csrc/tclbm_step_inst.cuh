@@ -236,47 +236,64 @@ cudaError_t BATCH_TMA_FN(int tx, unsigned grid, const BatchLattice* lats, const 
     return cudaGetLastError();
 }
 
-template <int KIND, bool MULTI, bool FAST = false>
-static cudaError_t launch_resident_kind(const ResLaunch& r, const DevParams& p0, const void* src, void* dst,
-                                        cudaStream_t s) {
-    DevParams p = p0;
-    p.parity = r.parity;
+// `fn` with the resident kernel of plan `r` for a lattice of parameters `p` and its dynamic
+// shared memory, the limit raised (always: the static arrays count towards the default too).
+template <int KIND, bool MULTI, bool FAST, class F>
+static cudaError_t resident_instance(F&& fn) {
     auto kernel = tclbm_resident<ST, KIND, MULTI, FAST>;
     const size_t smem = ResShape<KIND, MULTI>::SMEM;
-    // (always raised: the static arrays count towards the default limit too)
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(r.plan.gx * r.plan.gy), 1, 1);
-    cfg.blockDim = dim3((unsigned)r.plan.threads, 1, 1);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeCooperative;  // the CTAs wait for one another
-    attr[0].val.cooperative = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, kernel, p, static_cast<const ST*>(src), static_cast<ST*>(dst),
-                           static_cast<uint4*>(r.board), r.plan.gx, r.plan.gy, r.n, r.tag0, r.err);
-    if (e == cudaSuccess && p.rounding) {
-        tclbm_count_steps<<<1, 1, 0, s>>>(p, r.parity ^ (r.n & 1), (unsigned)r.n);
-        e = cudaGetLastError();
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    return e != cudaSuccess ? e : fn(kernel, smem);
+}
+template <class F>
+static cudaError_t with_resident_kernel(int kind, const ResPlan& plan, const DevParams& p, F&& fn) {
+    switch (kind) {
+        case RES_CORR:
+            return options_fast(p) ? resident_instance<RES_CORR, false, true>(fn)
+                                   : resident_instance<RES_CORR, false, false>(fn);
+        case RES_THERMAL:
+            return plan.multi ? resident_instance<RES_THERMAL, true, false>(fn)
+                              : resident_instance<RES_THERMAL, false, false>(fn);
+        default:
+            return plan.multi ? resident_instance<RES_ATHERMAL, true, false>(fn)
+                              : resident_instance<RES_ATHERMAL, false, false>(fn);
     }
-    return e;
 }
 
-cudaError_t RESIDENT_FN(const ResLaunch& r, const DevParams& p, const void* src, void* dst, cudaStream_t s) {
-    switch (r.kind) {
-        case RES_CORR:
-            return options_fast(p) ? launch_resident_kind<RES_CORR, false, true>(r, p, src, dst, s)
-                                   : launch_resident_kind<RES_CORR, false>(r, p, src, dst, s);
-        case RES_THERMAL:
-            return r.plan.multi ? launch_resident_kind<RES_THERMAL, true>(r, p, src, dst, s)
-                                : launch_resident_kind<RES_THERMAL, false>(r, p, src, dst, s);
-        default:
-            return r.plan.multi ? launch_resident_kind<RES_ATHERMAL, true>(r, p, src, dst, s)
-                                : launch_resident_kind<RES_ATHERMAL, false>(r, p, src, dst, s);
+cudaError_t RESIDENT_FN(const ResLaunch& r, const DevParams& p0, const void* src, void* dst, cudaStream_t s) {
+    DevParams p = p0;
+    p.parity = r.parity;
+    return with_resident_kernel(r.kind, r.plan, p, [&](auto kernel, size_t smem) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)(r.plan.gx * r.plan.gy), 1, 1);
+        cfg.blockDim = dim3((unsigned)r.plan.threads, 1, 1);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = s;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeCooperative;  // the CTAs wait for one another
+        attr[0].val.cooperative = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, p, static_cast<const ST*>(src), static_cast<ST*>(dst),
+                                           static_cast<uint4*>(r.board), r.plan.gx, r.plan.gy, r.n, r.tag0, r.err);
+        if (e == cudaSuccess && p.rounding) {
+            tclbm_count_steps<<<1, 1, 0, s>>>(p, r.parity ^ (r.n & 1), (unsigned)r.n);
+            e = cudaGetLastError();
+        }
+        return e;
+    });
+}
+
+int RESIDENT_OCC_FN(int kind, const ResPlan& plan, const DevParams& p) {
+    int n = 0;
+    const cudaError_t e = with_resident_kernel(kind, plan, p, [&](auto kernel, size_t smem) {
+        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, plan.threads, smem);
+    });
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
     }
+    return n;
 }
 
 int BATCH_OCC_FN(int tx, int kind) {

@@ -818,3 +818,45 @@ def test_new_fields_in_a_captured_graph_continue_the_draws(T):
     exp = lat.populations()
     lat.close()
     assert np.array_equal(got[0], exp[0]) and np.array_equal(got[1], exp[1])
+
+
+def test_lattices_on_several_streams_share_the_device(T):
+    # a resident launch that fills the device is for a device with one stream in use; small
+    # lattices stay resident beside others.  The states do not depend on it, bit for bit
+    import torch
+
+    def lattice(make):
+        stream = torch.cuda.Stream()
+        with torch.cuda.stream(stream):
+            return T.Lattice(*make(), stream=stream.cuda_stream)
+
+    def resident(lat):
+        return "tclbm_resident" in lat.describe()
+
+    def wide():
+        return W.rayleigh_benard(256, 128, seed=21)
+
+    def narrow():
+        return W.couette(8, 64)
+
+    a = lattice(wide)
+    assert resident(a)
+    a.step(30)  # resident
+    b, c = lattice(narrow), lattice(wide)
+    assert not resident(a) and not resident(c) and resident(b)
+    for lat in (a, b, c):
+        lat.step(40)
+    b.close()
+    assert not resident(a)
+    c.set_stream(a.stream)  # one stream again
+    assert resident(a) and resident(c)
+    c.step(30)
+    batch = T.Batch([c], stream=torch.cuda.Stream().cuda_stream)
+    assert not resident(a)
+    batch.close()
+    assert resident(a)
+    got = [lat.populations() for lat in (a, c)]
+    c.close()
+    a.close()
+    for f, h in got:
+        assert np.array_equal(f, got[0][0]) and np.array_equal(h, got[0][1])
