@@ -247,6 +247,12 @@ tclbm_status tclbm_test_skip_row(tclbm_lattice* lat, int32_t row);
  * EINVAL on n < 0 or NULL arrays with n > 0. */
 tclbm_status tclbm_test_rcp(const float* x, float* y, int64_t n, void* stream);
 
+/* Test hook for the division of the field conversions (no counterpart in the paper): y[i] =
+ * a[i] / x[i] as moments and diagnostics form it, within one unit in the last place and equal
+ * where the quotient is zero, infinite or NaN; n doubles at device pointers.  Queued on
+ * `stream`, which it synchronises.  EINVAL on n < 0 or NULL arrays with n > 0. */
+tclbm_status tclbm_test_div(const double* a, const double* x, double* y, int64_t n, void* stream);
+
 /* Test hook for the node order of the field conversions (no counterpart in the paper; host
  * code, no device work): x[k], y[k] = column and row, in a lattice nx wide, of node
  * first + k * stride as a thread of the conversion kernels counts them, for k < count.

@@ -528,7 +528,7 @@ __global__ void __launch_bounds__(kDiagBlock) diag_kernel(const DevParams p, con
     if (p.force_kind == FORCE_TAYLOR_GREEN) {
         acc[1] = __fma_rn(0.5 * (double)p.famp, Fxs, acc[1]);
         acc[2] = __fma_rn(0.5 * (double)p.famp, Fys, acc[2]);
-    } else {
+    } else if (p.force_kind == FORCE_ACCEL) {
         acc[1] = __fma_rn(0.5 * (double)p.ax, acc[0], acc[1]);
         acc[2] = __fma_rn(0.5 * (double)p.ay, acc[0], acc[2]);
     }
@@ -1034,6 +1034,13 @@ __global__ void rcp_kernel(const float* __restrict__ x, float* __restrict__ y, l
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
         y[i] = tclbm::rcp(x[i]);
 }
+
+// The quotient the field conversions take.
+__global__ void div_kernel(const double* __restrict__ a, const double* __restrict__ x, double* __restrict__ y,
+                           long long n) {
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+        y[i] = div_d(a[i], x[i], rcp_d(x[i]));
+}
 }  // namespace
 
 tclbm_status tclbm_test_rcp(const float* x, float* y, int64_t n, void* stream) {
@@ -1041,6 +1048,16 @@ tclbm_status tclbm_test_rcp(const float* x, float* y, int64_t n, void* stream) {
     if (n == 0) return TCLBM_OK;
     cudaStream_t s = (cudaStream_t)stream;
     rcp_kernel<<<grid_for(n, 256), 256, 0, s>>>(x, y, n);
+    CK(cudaGetLastError());
+    CK(cudaStreamSynchronize(s));
+    return TCLBM_OK;
+}
+
+tclbm_status tclbm_test_div(const double* a, const double* x, double* y, int64_t n, void* stream) {
+    if (n < 0 || (n > 0 && (!a || !x || !y))) return fail(TCLBM_EINVAL, "a, x, y must be device arrays of n >= 0 doubles");
+    if (n == 0) return TCLBM_OK;
+    cudaStream_t s = (cudaStream_t)stream;
+    div_kernel<<<grid_for(n, 256), 256, 0, s>>>(a, x, y, n);
     CK(cudaGetLastError());
     CK(cudaStreamSynchronize(s));
     return TCLBM_OK;

@@ -99,20 +99,32 @@ __device__ __forceinline__ Sum3 sum_of(const float (&v)[N]) {
     return p;
 }
 
-// 1/x from the FP32 approximation and one third-order step (relative error near 2^-53).
+// Whether |x| is in 2^-63 .. 2^63, where the reciprocal below starts from FP32.
+__device__ __forceinline__ bool rcp_range(double x) {
+    return ((unsigned)__double2hiint(x) & 0x7fffffffu) - 0x3c000000u < 0x07f00000u;
+}
+
+// 1/x: the FP32 approximation (2^-23) and one third-order iteration of Newton's kind,
+// y (1 + e + e^2) with e = 1 - x y, whose own error is e^3; plain division outside rcp_range().
 __device__ __forceinline__ double rcp_d(double x) {
-    const unsigned m = (unsigned)__double2hiint(x) & 0x7fffffffu;
-    if (m - 0x3c000000u >= 0x07f00000u) return 1.0 / x;  // outside 2^-63 .. 2^63
+    if (!rcp_range(x)) return 1.0 / x;
     float r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d2f(x)));
     const double y = f2d(r), e = __fma_rn(-x, y, 1.0);
     return __fma_rn(y, __fma_rn(e, e, e), y);
 }
 
-// a / x, r = rcp_d(x): one correction of the quotient by its remainder.
+// a / x, r = rcp_d(x): the quotient corrected by its remainder (P. Markstein's method; within
+// one unit in the last place), where x, the quotient and the remainder are ordinary numbers;
+// zeros, infinities, NaN and the ends of the exponent range divide plainly.
 __device__ __forceinline__ double div_d(double a, double x, double r) {
     const double q = a * r;
-    return __fma_rn(__fma_rn(-q, x, a), r, q);
+    if (rcp_range(x)) {
+        if (((unsigned)__double2hiint(q) & 0x7fffffffu) - 0x0ad00000u < 0x6d800000u)  // 2^-850 .. 2^902
+            return __fma_rn(__fma_rn(-q, x, a), r, q);
+        if ((((unsigned)__double2hiint(a) & 0x7fffffffu) | (unsigned)__double2loint(a)) == 0) return q;
+    }
+    return a / x;
 }
 
 // Sums of a node's deviations: rho - 1, the momentum without the force, sum h_bar less its
@@ -143,7 +155,7 @@ __device__ __forceinline__ NodeFields node_velocity(const DevParams& p, const No
         const double a = 0.5 * f2d(p.famp);
         jx = __fma_rn(a * f2d(p.sx[x]), f2d(p.sy[y]), jx);
         jy = __fma_rn(a * f2d(p.cx[x]), f2d(p.cy[y]), jy);
-    } else {
+    } else if (p.force_kind == FORCE_ACCEL) {
         jx = __fma_rn(0.5 * f2d(p.ax), n.rho, jx);
         jy = __fma_rn(0.5 * f2d(p.ay), n.rho, jy);
     }
@@ -158,11 +170,11 @@ __device__ __forceinline__ double node_temperature(const DevParams& p, const Nod
                                                    int y) {
     if (!THERMAL) return p.T0d;
     if (p.work) {  // rho E = sum h_bar + F.u / 2
-        double Fx, Fy;
+        double Fx = 0.0, Fy = 0.0;
         if (p.force_kind == FORCE_TAYLOR_GREEN) {
             Fx = f2d(p.famp) * f2d(p.sx[x]) * f2d(p.sy[y]);
             Fy = f2d(p.famp) * f2d(p.cx[x]) * f2d(p.cy[y]);
-        } else {
+        } else if (p.force_kind == FORCE_ACCEL) {
             Fx = n.rho * f2d(p.ax);
             Fy = n.rho * f2d(p.ay);
         }

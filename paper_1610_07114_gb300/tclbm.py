@@ -100,6 +100,8 @@ _lib.tclbm_test_skip_row.argtypes = [_vp, ctypes.c_int32]
 _lib.tclbm_test_skip_row.restype = ctypes.c_int
 _lib.tclbm_test_rcp.argtypes = [_vp, _vp, ctypes.c_int64, _vp]
 _lib.tclbm_test_rcp.restype = ctypes.c_int
+_lib.tclbm_test_div.argtypes = [_vp, _vp, _vp, ctypes.c_int64, _vp]
+_lib.tclbm_test_div.restype = ctypes.c_int
 _i32p = ctypes.POINTER(ctypes.c_int32)
 _lib.tclbm_test_node_walk.argtypes = [ctypes.c_uint32, ctypes.c_uint32, ctypes.c_int32, ctypes.c_int64, _i32p, _i32p]
 _lib.tclbm_test_node_walk.restype = ctypes.c_int
@@ -215,6 +217,10 @@ def tclbm_test_skip_row(h, row):
 
 def tclbm_test_rcp(x, y, n, stream=None):
     _check(_lib.tclbm_test_rcp(x, y, int(n), stream), "tclbm_test_rcp")
+
+
+def tclbm_test_div(a, x, y, n, stream=None):
+    _check(_lib.tclbm_test_div(a, x, y, int(n), stream), "tclbm_test_div")
 
 
 def tclbm_test_node_walk(first, stride, nx, count):

@@ -196,3 +196,59 @@ def test_moments_of_given_populations_to_the_last_digits(T, force, amp):
     scale = max(float(np.abs(ux).max()), float(np.abs(uy).max()))
     assert float(np.abs(m["ux"] - ux).max()) <= 2 * eps * scale + 12 * 2.0 ** -55 * (amp < 1e-6)
     assert float(np.abs(m["uy"] - uy).max()) <= 2 * eps * scale + 12 * 2.0 ** -55 * (amp < 1e-6)
+
+
+def test_division_over_the_whole_exponent_range(T):
+    # the quotient of the field conversions against IEEE division: one unit in the last place
+    # (a corrected quotient misses the rounded one by at most that), equal for zeros, infinities,
+    # NaN, subnormal numbers and where it overflows
+    import torch
+
+    rng = np.random.default_rng(65)
+    n = 1 << 18
+    sign = rng.choice([-1.0, 1.0], n)
+    wide = sign * np.ldexp(1 + rng.random(n), rng.integers(-1074, 1024, n).astype(np.int32))
+    near = sign * np.ldexp(1 + rng.random(n), rng.integers(-66, 66, n).astype(np.int32))
+    special = np.array([0.0, -0.0, 1.0, -1.0, np.inf, -np.inf, np.nan, 5e-324, -5e-324, 2.0 ** -1022, 1.7e308, -1.7e308,
+                        2.0 ** -63, 2.0 ** 64, np.nextafter(2.0 ** 64, 0), 2.0 ** -64, 1e-300, 1e300, 1 / 3, 2.0 ** -850])
+    sa, sx = (g.ravel() for g in np.meshgrid(special, np.concatenate([special, near[:400], wide[:400]])))
+    a = np.concatenate([wide, near, near, sa, sx])
+    x = np.concatenate([near, rng.permutation(near), rng.permutation(wide), sx, sa])
+    dev = [torch.as_tensor(v, device="cuda") for v in (a, x)]
+    y = torch.empty_like(dev[0])
+    T.tclbm_test_div(dev[0].data_ptr(), dev[1].data_ptr(), y.data_ptr(), a.size)
+    got = y.cpu().numpy()
+    with np.errstate(all="ignore"):
+        want = a / x
+    plain = ~np.isfinite(want) | (np.abs(want) < 2.0 ** -851) | (np.abs(x) < 2.0 ** -63) | (np.abs(x) >= 2.0 ** 64)
+    assert np.array_equal(got[plain], want[plain], equal_nan=True)
+    assert np.array_equal(np.signbit(got[want == 0]), np.signbit(want[want == 0]))
+    err = np.abs(got[~plain] - want[~plain]) / np.spacing(np.abs(want[~plain]))
+    assert err.max() <= 1.0, err.max()
+    with pytest.raises(T.TclbmError):
+        T.tclbm_test_div(None, None, None, 5)
+
+
+@pytest.mark.parametrize("thermal", [True, False])
+def test_moments_of_infinite_and_of_zero_density(T, thermal):
+    # one infinite population, and populations whose sum is exactly zero: the quotients by the
+    # density are those of plain arithmetic (0, infinite or NaN), at these nodes alone
+    case, _ = W.random_periodic(40, 6, seed=66, force="none", correction=thermal)
+    case = dict(case, thermal=thermal)
+    lat = T.Lattice(case)
+    f, h = lat.populations()
+    h = np.zeros_like(f) if h is None else h
+    f[:, 2, 3] = [np.inf, 0, 0, 0, 0, 0, 0, 0, 0]
+    f[:, 4, 5] = [0, 2.0 ** -10, 2.0 ** -10, -2.0 ** -10, -2.0 ** -10, 0, 0, 0, 0]
+    lat.set_populations(f, h if thermal else None)
+    f, h2 = lat.populations()
+    m = lat.moments()
+    lat.close()
+    assert f[0, 2, 3] == np.inf and f[:, 4, 5].sum() == 0.0
+    assert m["rho"][2, 3] == np.inf and m["ux"][2, 3] == 0.0 and m["uy"][2, 3] == 0.0
+    assert m["rho"][4, 5] == 0.0 and m["ux"][4, 5] == np.inf and m["uy"][4, 5] == np.inf
+    if thermal:
+        assert m["T"][2, 3] == 0.0 and np.isnan(m["T"][4, 5])
+    for k in m:
+        bad = ~np.isfinite(m[k])
+        assert bad.sum() == bad[2, 3] + bad[4, 5]
