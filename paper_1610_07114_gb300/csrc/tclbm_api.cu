@@ -464,13 +464,12 @@ __global__ void moments_kernel(const DevParams p, const ST* __restrict__ src, do
         const int x = w.x, y = w.y;
         float fv[9], hv[9];
         load_node<THERMAL, ST>(p, src, x, y, fv, hv);
-        const NodeSums s = node_sums<THERMAL>(fv, hv);
+        const NodeTotals s = node_totals<THERMAL>(p, node_sums<THERMAL>(fv, hv), fv, hv);
         const NodeFields v = node_velocity(p, s, x, y);
-        const double sh = THERMAL ? sum_value(p.hrest, s.sdh) : 0.0;
         rho[i] = v.rho;
         ux[i] = v.ux;
         uy[i] = v.uy;
-        T[i] = node_temperature<THERMAL>(p, v, sh, THERMAL ? __fma_rn(v.ux, v.ux, v.uy * v.uy) : 0.0, x, y);
+        T[i] = node_temperature<THERMAL>(p, v, s.sh, THERMAL ? __fma_rn(v.ux, v.ux, v.uy * v.uy) : 0.0, x, y);
     }
 }
 
@@ -489,8 +488,9 @@ __global__ void __launch_bounds__(kDiagBlock) diag_kernel(const DevParams p, con
     double acc[TCLBM_NDIAG] = {0, 0, 0, 0, 0, 0, 0, 0};
     const long long n = (long long)p.nx * p.ny;
     // the linear sums stay FP32 error-free sums of deviations until the thread's last node
+    // (where a node's are narrow; the others enter acc at once)
     Running drho, jx, jy, sdh;
-    double nodes = 0, Fxs = 0, Fys = 0;  // nodes seen, and their Taylor-Green forces
+    double nodes = 0, Fxs = 0, Fys = 0;  // narrow nodes seen; the Taylor-Green forces of all
     NodeWalk w(blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x, p.nx);
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x, w.next(p.nx)) {
@@ -498,21 +498,26 @@ __global__ void __launch_bounds__(kDiagBlock) diag_kernel(const DevParams p, con
         float fv[9], hv[9];
         load_node<THERMAL, ST>(p, src, x, y, fv, hv);
         const NodeSums s = node_sums<THERMAL>(fv, hv);
-        const NodeFields v = node_velocity(p, s, x, y);
+        const NodeTotals total = node_totals<THERMAL>(p, s, fv, hv);
+        const NodeFields v = node_velocity(p, total, x, y);
         const double uu = __fma_rn(v.ux, v.ux, v.uy * v.uy);
-        drho.add(s.drho);
-        jx.add(s.jx);
-        jy.add(s.jy);
+        if (s.narrow()) {
+            drho.add(s.drho);
+            jx.add(s.jx);
+            jy.add(s.jy);
+            if (THERMAL) sdh.add(s.sdh);
+            nodes += 1.0;
+        } else {
+            acc[0] += total.rho;
+            acc[1] += total.jx;
+            acc[2] += total.jy;
+            acc[3] += total.sh;
+        }
         if (p.force_kind == FORCE_TAYLOR_GREEN) {
             Fxs = __fma_rn(f2d(p.sx[x]), f2d(p.sy[y]), Fxs);
             Fys = __fma_rn(f2d(p.cx[x]), f2d(p.cy[y]), Fys);
         }
-        double t = p.T0d;
-        if (THERMAL) {
-            sdh.add(s.sdh);
-            t = node_temperature<THERMAL>(p, v, sum_value(p.hrest, s.sdh), uu, x, y);
-        }
-        nodes += 1.0;
+        const double t = node_temperature<THERMAL>(p, v, total.sh, uu, x, y);
         acc[4] = __fma_rn(v.rho, uu, acc[4]);
         acc[5] = __fma_rn(v.uy, t - T_ref, acc[5]);
         if (usnap) {
@@ -522,9 +527,9 @@ __global__ void __launch_bounds__(kDiagBlock) diag_kernel(const DevParams p, con
         acc[7] += uu;
     }
     // sum rho, sum (j + F/2), sum h_bar and the kinetic energy of this thread's nodes
-    acc[0] = nodes + drho.value();
-    acc[1] = jx.value();
-    acc[2] = jy.value();
+    acc[0] += nodes + drho.value();
+    acc[1] += jx.value();
+    acc[2] += jy.value();
     if (p.force_kind == FORCE_TAYLOR_GREEN) {
         acc[1] = __fma_rn(0.5 * (double)p.famp, Fxs, acc[1]);
         acc[2] = __fma_rn(0.5 * (double)p.famp, Fys, acc[2]);
@@ -532,7 +537,7 @@ __global__ void __launch_bounds__(kDiagBlock) diag_kernel(const DevParams p, con
         acc[1] = __fma_rn(0.5 * (double)p.ax, acc[0], acc[1]);
         acc[2] = __fma_rn(0.5 * (double)p.ay, acc[0], acc[2]);
     }
-    acc[3] = THERMAL ? __fma_rn(nodes, p.hrest, sdh.value()) : 0.0;
+    if (THERMAL) acc[3] += __fma_rn(nodes, p.hrest, sdh.value());
     acc[4] *= 0.5;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
@@ -569,7 +574,7 @@ __global__ void snapshot_kernel(const DevParams p, const ST* __restrict__ src, f
         const int x = w.x, y = w.y;
         float fv[9], hv[9];
         load_node<THERMAL, ST>(p, src, x, y, fv, hv);
-        const NodeFields v = node_velocity(p, node_sums<false>(fv, hv), x, y);
+        const NodeFields v = node_velocity(p, node_totals<false>(p, node_sums<false>(fv, hv), fv, hv), x, y);
         usnap[2 * i] = d2f(v.ux);
         usnap[2 * i + 1] = d2f(v.uy);
     }

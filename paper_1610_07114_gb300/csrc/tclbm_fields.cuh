@@ -80,15 +80,9 @@ __device__ __forceinline__ void sum_add(Sum3& p, float v) {
     two_sum(p.mid, e, p.mid, e);
     p.lo = __fadd_rn(p.lo, e);
 }
-// base + sum (an infinite or undefined sum has no error terms)
-__device__ __forceinline__ double sum_value(double base, const Sum3& p) {
-    if (!(fabsf(p.hi) <= 3.402823466e38f)) return base + (double)p.hi;
-    return base + f2d(p.hi) + (f2d(p.mid) + f2d(p.lo));
-}
-__device__ __forceinline__ double sum_value(const Sum3& p) {
-    if (!(fabsf(p.hi) <= 3.402823466e38f)) return (double)p.hi;
-    return f2d(p.hi) + (f2d(p.mid) + f2d(p.lo));
-}
+// base + sum, for sums that are narrow()
+__device__ __forceinline__ double sum_value(double base, const Sum3& p) { return base + f2d(p.hi) + (f2d(p.mid) + f2d(p.lo)); }
+__device__ __forceinline__ double sum_value(const Sum3& p) { return f2d(p.hi) + (f2d(p.mid) + f2d(p.lo)); }
 template <int N>
 __device__ __forceinline__ Sum3 sum_of(const float (&v)[N]) {
     Sum3 p;
@@ -131,6 +125,11 @@ __device__ __forceinline__ double div_d(double a, double x, double r) {
 // rest value.
 struct NodeSums {
     Sum3 drho, jx, jy, sdh;
+    // Whether they can be carried in FP32 (and summed over the 2^15 nodes a thread sees of the
+    // largest lattice): not where a sum comes near FP32's range, is infinite or undefined.
+    __device__ __forceinline__ bool narrow() const {
+        return fabsf(drho.hi) + fabsf(jx.hi) + fabsf(jy.hi) + fabsf(sdh.hi) < 7.9e28f;  // 2^96
+    }
 };
 template <bool THERMAL>
 __device__ __forceinline__ NodeSums node_sums(const float (&f)[9], const float (&h)[9]) {
@@ -138,19 +137,45 @@ __device__ __forceinline__ NodeSums node_sums(const float (&f)[9], const float (
     s.drho = sum_of(f);
     s.jx = sum_of({f[1], -f[3], f[5], -f[6], f[8], -f[7]});
     s.jy = sum_of({f[2], -f[4], f[5], -f[7], f[6], -f[8]});
-    if (THERMAL) s.sdh = sum_of(h);
+    if (THERMAL)
+        s.sdh = sum_of(h);
+    else
+        s.sdh = Sum3{0.0f, 0.0f, 0.0f};
     return s;
+}
+
+// The sums themselves: rho, the momentum without the force, sum h_bar; in plain FP64 arithmetic
+// where the FP32 parts do not hold them.
+struct NodeTotals {
+    double rho, jx, jy, sh;
+};
+template <bool THERMAL>
+__device__ __forceinline__ NodeTotals node_totals(const DevParams& p, const NodeSums& s, const float (&f)[9],
+                                                  const float (&h)[9]) {
+    if (s.narrow())
+        return NodeTotals{sum_value(1.0, s.drho), sum_value(s.jx), sum_value(s.jy), THERMAL ? sum_value(p.hrest, s.sdh) : 0.0};
+    const int ex[9] = {0, 1, 0, -1, 0, 1, -1, -1, 1}, ey[9] = {0, 0, 1, 0, -1, 1, 1, -1, -1};
+    NodeTotals t = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+    for (int q = 0; q < 9; ++q) {
+        const double fq = p.fbase_d[q] + (double)f[q];
+        t.rho += fq;
+        if (ex[q] != 0) t.jx += fq * ex[q];
+        if (ey[q] != 0) t.jy += fq * ey[q];
+        if (THERMAL) t.sh += p.hbase_d[q] + (double)h[q];
+    }
+    return t;
 }
 
 // rho and u of Eq. 20 from the sums (Fx, Fy: the Taylor-Green force, else unused).
 struct NodeFields {
     double rho, irho, ux, uy;
 };
-__device__ __forceinline__ NodeFields node_velocity(const DevParams& p, const NodeSums& s, int x, int y) {
+__device__ __forceinline__ NodeFields node_velocity(const DevParams& p, const NodeTotals& s, int x, int y) {
     NodeFields n;
-    n.rho = sum_value(1.0, s.drho);
+    n.rho = s.rho;
     n.irho = rcp_d(n.rho);
-    double jx = sum_value(s.jx), jy = sum_value(s.jy);
+    double jx = s.jx, jy = s.jy;
     if (p.force_kind == FORCE_TAYLOR_GREEN) {
         const double a = 0.5 * f2d(p.famp);
         jx = __fma_rn(a * f2d(p.sx[x]), f2d(p.sy[y]), jx);
@@ -183,7 +208,7 @@ __device__ __forceinline__ double node_temperature(const DevParams& p, const Nod
     return p.inv_bR2 * __fma_rn(-0.5, uu, div_d(sh, n.rho, n.irho));
 }
 
-// A running sum of FP32 values in three parts (error-free to far below FP64's rounding).
+// A running sum of narrow() FP32 values in three parts (error-free to far below FP64's rounding).
 struct Running {
     float a = 0.0f, b = 0.0f, c = 0.0f;
     __device__ __forceinline__ void add(float v) {
@@ -196,9 +221,7 @@ struct Running {
         add(p.hi);
         add(p.mid);  // (lo is below 2^-48 of a deviation and 2^-72 of the sum it would enter)
     }
-    __device__ __forceinline__ double value() const {
-        return fabsf(a) <= 3.402823466e38f ? (f2d(c) + f2d(b)) + f2d(a) : (double)a;
-    }
+    __device__ __forceinline__ double value() const { return (f2d(c) + f2d(b)) + f2d(a); }
 };
 
 }  // namespace tclbm

@@ -252,3 +252,45 @@ def test_moments_of_infinite_and_of_zero_density(T, thermal):
     for k in m:
         bad = ~np.isfinite(m[k])
         assert bad.sum() == bad[2, 3] + bad[4, 5]
+
+
+@pytest.mark.parametrize("thermal", [True, False])
+def test_sums_beyond_the_range_of_fp32(T, thermal):
+    # populations that FP32 holds but whose sums it does not: moments and global sums are those of
+    # FP64 arithmetic, nine and a few thousand terms of 2^-53 each
+    nx, ny = 64, 48
+    case, _ = W.random_periodic(nx, ny, seed=67, force="none", correction=thermal)
+    case = dict(case, thermal=thermal)
+    lat = T.Lattice(case)
+    f, h = lat.populations()
+    rng = np.random.default_rng(68)
+    f[:, ::5, ::7] += 3e38 * rng.uniform(0.5, 1.0, f[:, ::5, ::7].shape)
+    f[:, 1::5, ::7] *= 1e30 * rng.uniform(0.5, 1.0, f[:, 1::5, ::7].shape)
+    if thermal:
+        h[:, 2::5, ::7] += 3e38 * rng.uniform(0.5, 1.0, h[:, 2::5, ::7].shape)
+    lat.set_populations(f, h)
+    f, h = lat.populations()
+    m, d = lat.moments(), lat.diagnostics()
+    lat.snapshot_velocity()
+    again = lat.diagnostics()
+    p = lat.params
+    lat.close()
+    ex, ey = (0, 1, 0, -1, 0, 1, -1, -1, 1), (0, 0, 1, 0, -1, 1, 1, -1, -1)
+    rho = f.sum(0)
+    jx, jy = sum(e * v for e, v in zip(ex, f)), sum(e * v for e, v in zip(ey, f))
+    assert rho.max() > 1e39 and np.isfinite(rho).all()
+    scale = np.abs(f).sum(0)
+    assert (np.abs(m["rho"] - rho) <= 2.0 ** -49 * scale).all()
+    for k, j in (("ux", jx), ("uy", jy)):
+        assert (np.abs(m[k] - j / rho) <= 2.0 ** -49 * scale / np.abs(rho)).all()
+    tol = 2.0 ** -41
+    for got, want, mag in ((d[0], rho.sum(), scale.sum()), (d[1], jx.sum(), scale.sum()), (d[2], jy.sum(), scale.sum())):
+        assert abs(got - want) <= tol * mag
+    uu = (jx / rho) ** 2 + (jy / rho) ** 2
+    assert abs(d[7] - uu.sum()) <= tol * uu.sum()
+    if thermal:
+        assert abs(d[3] - h.sum()) <= tol * np.abs(h).sum()
+        c = 2.0 / (2.0 / (p.gamma - 1.0) * p.R)
+        E = h.sum(0) / rho
+        assert (np.abs(m["T"] - c * (E - uu / 2)) <= 2.0 ** -47 * c * (np.abs(h).sum(0) / rho + uu)).all()
+    assert abs(again[6]) <= 2.0 ** -40 * uu.sum() and again[7] == d[7]  # (the snapshot is FP32)
