@@ -240,6 +240,13 @@ const char* tclbm_describe(const tclbm_lattice* lat);
  * it).  row = -1 turns the hook off.  EINVAL for other rows. */
 tclbm_status tclbm_test_skip_row(tclbm_lattice* lat, int32_t row);
 
+/* Test hook for failed launches (no counterpart in the paper): of the step launches (or
+ * resident runs) that calls on this thread make from now on, the one after `after` others is
+ * not made and reported as failed (TCLBM_ECUDA).  The steps launched before it are taken and
+ * counted: tclbm_steps_done() says how many, tclbm_batch_steps_done() how many every lattice
+ * of a batch has taken.  after = -1 turns the hook off.  EINVAL for other values below 0. */
+tclbm_status tclbm_test_fail_launch(int64_t after);
+
 /* Test hook for the collision's reciprocal (no counterpart in the paper): y[i] = the
  * reciprocal the step kernels take of R T, mu/p + 1/2 and mu/(p Pr) + 1/2 (the hardware
  * approximation refined by one Newton step), for n floats at device pointers x, y.

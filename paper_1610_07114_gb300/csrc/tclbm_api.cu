@@ -29,7 +29,10 @@ using namespace tclbm;
 
 namespace {
 thread_local char g_err[512] = "";
+thread_local int64_t g_refuse_in = -1;  // test hook: step launches left before one is refused
 }  // namespace
+
+bool tclbm::refuse_launch() { return g_refuse_in >= 0 && g_refuse_in-- == 0; }
 
 tclbm_status tclbm::fail(tclbm_status st, const char* fmt, ...) {
     va_list ap;
@@ -668,7 +671,9 @@ tclbm_status launch_steps(tclbm_lattice* L, int64_t n) {
     const bool tickets = L->kernel == KERNEL_TMA && L->prm.thermal && L->prm.correction;
     const bool chain = n > 1 && chainable(L) && !capturing(L->stream);
     const int first = L->cur;
-    for (int64_t s = 0; s < n; ++s) {
+    tclbm_status st = TCLBM_OK;
+    int64_t s = 0;
+    for (; s < n; ++s) {
         StepLaunch k = step_launch(L, L->cur);
         if (tickets) {
             k.seg_done = L->seg_done;
@@ -680,19 +685,24 @@ tclbm_status launch_steps(tclbm_lattice* L, int64_t n) {
             k.ctr_copy = first;
             k.ctr_add = (unsigned)s;
         }
-        const cudaError_t e = launch_step_kernel(L->prm.storage, k, L->dp, L->buf[L->cur], L->buf[L->cur ^ 1], L->stream);
-        if (e != cudaSuccess) return cuda_fail(e, "step kernel launch");
+        const cudaError_t e = refuse_launch() ? cudaErrorLaunchOutOfResources
+                                              : launch_step_kernel(L->prm.storage, k, L->dp, L->buf[L->cur],
+                                                                   L->buf[L->cur ^ 1], L->stream);
+        if (e != cudaSuccess) {
+            st = cuda_fail(e, "step kernel launch");
+            break;
+        }
         L->cur ^= 1;
         ++L->steps;
     }
-    if (chain && L->dp.rounding) {
+    if (chain && L->dp.rounding && s > 0) {  // also after a failure: the steps that were launched count
         DevParams p = L->dp;
         p.parity = first;
-        tclbm_count_steps<<<1, 1, 0, L->stream>>>(p, L->cur, (unsigned)n);
+        tclbm_count_steps<<<1, 1, 0, L->stream>>>(p, L->cur, (unsigned)s);
         const cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return cuda_fail(e, "step counter");
+        if (e != cudaSuccess && st == TCLBM_OK) st = cuda_fail(e, "step counter");
     }
-    return TCLBM_OK;
+    return st;
 }
 
 // Steps of one resident launch at most (1.5 to 6 ms, which work of other streams may have to
@@ -762,7 +772,9 @@ tclbm_status resident_steps(tclbm_lattice* L, int64_t n, int64_t& done) {
         r.board = L->board;
         r.err = L->err;
         const int to = L->cur ^ (int)(k & 1);  // the copy that k launches would end in
-        const cudaError_t e = launch_resident(L->prm.storage, r, L->dp, L->buf[L->cur], L->buf[to], L->stream);
+        const cudaError_t e = refuse_launch()
+                                  ? cudaErrorLaunchOutOfResources
+                                  : launch_resident(L->prm.storage, r, L->dp, L->buf[L->cur], L->buf[to], L->stream);
         if (e == cudaErrorCooperativeLaunchTooLarge) {  // fewer multiprocessors than the device has are ours
             cudaGetLastError();
             L->res_state = -1;
@@ -1030,6 +1042,12 @@ tclbm_status tclbm_test_skip_row(tclbm_lattice* L, int32_t row) {
         cudaGraphExecDestroy(L->graph);
         L->graph = nullptr;
     }
+    return TCLBM_OK;
+}
+
+tclbm_status tclbm_test_fail_launch(int64_t after) {
+    if (after < -1) return fail(TCLBM_EINVAL, "after must be >= -1");
+    g_refuse_in = after;
     return TCLBM_OK;
 }
 

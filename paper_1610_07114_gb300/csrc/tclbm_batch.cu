@@ -51,6 +51,7 @@ struct tclbm_batch {
     int gen = 0;
     std::vector<BatchLattice> h_lats;  // last uploaded descriptors
     int64_t steps = 0;                 // batch steps taken (parity of the next launch)
+    int64_t done[4] = {0, 0, 0, 0};    // steps of each group launched by the current call
     bool items_valid = false;
     // what the uploaded work list was built from: (nx, ny, variant) per lattice in list
     // order and the shape; a handle's address says nothing (a destroyed lattice's
@@ -283,8 +284,9 @@ cudaError_t launch_group(const tclbm_batch* B, int g, int parity, cudaStream_t s
 // n steps from parity `parity`, ordered on `s`.  The groups hold different lattices, so each
 // runs its own chain of launches beside the others: a group of a few narrow lattices takes
 // about as long as its rows are deep (40 us for 64 x 32 lattices in 16-row strips) and
-// would otherwise leave the device idle once a step.
-tclbm_status launch_chain(tclbm_batch* B, int64_t n, int parity, cudaStream_t s) {
+// would otherwise leave the device idle once a step.  `done` (if given): steps launched of
+// each group, which differ by one at most after a failure.
+tclbm_status launch_chain(tclbm_batch* B, int64_t n, int parity, cudaStream_t s, int64_t* done) {
     int groups[4], ng = 0;
     for (int g : {kGroupTma, (int)BATCH_THERMAL_CORR, (int)BATCH_THERMAL, (int)BATCH_ATHERMAL})
         if (B->count[g] > 0) groups[ng++] = g;
@@ -301,7 +303,11 @@ tclbm_status launch_chain(tclbm_batch* B, int64_t n, int parity, cudaStream_t s)
     }
     cudaError_t e = cudaSuccess;
     for (int64_t k = 0; k < n && e == cudaSuccess; ++k)
-        for (int i = 0; i < ng && e == cudaSuccess; ++i) e = launch_group(B, groups[i], (int)((parity + k) & 1), on[i]);
+        for (int i = 0; i < ng && e == cudaSuccess; ++i) {
+            e = refuse_launch() ? cudaErrorLaunchOutOfResources
+                                : launch_group(B, groups[i], (int)((parity + k) & 1), on[i]);
+            if (e == cudaSuccess && done) ++done[groups[i]];
+        }
     for (int i = 1; i < ng; ++i) {  // also after a failed launch: nothing may outlive the batch stream's order
         const cudaError_t r = cudaEventRecord(B->join[i - 1], on[i]);
         const cudaError_t w = r == cudaSuccess ? cudaStreamWaitEvent(s, B->join[i - 1], 0) : r;
@@ -310,10 +316,19 @@ tclbm_status launch_chain(tclbm_batch* B, int64_t n, int parity, cudaStream_t s)
     return e == cudaSuccess ? TCLBM_OK : cuda_fail(e, "batched step kernel launch");
 }
 
+// Steps that every group present has launched.
+int64_t steps_of_all(const tclbm_batch* B) {
+    int64_t n = INT64_MAX;
+    for (int g = 0; g < 4; ++g)
+        if (B->count[g] > 0) n = std::min(n, B->done[g]);
+    return n;
+}
+
 tclbm_status launch_batch_steps(tclbm_batch* B, int64_t n) {
     if (n <= 0) return TCLBM_OK;
-    tclbm_status st = launch_chain(B, n, (int)(B->steps & 1), B->stream);
-    if (st == TCLBM_OK) B->steps += n;
+    const int64_t before = steps_of_all(B);
+    const tclbm_status st = launch_chain(B, n, (int)(B->steps & 1), B->stream, B->done);
+    B->steps += steps_of_all(B) - before;
     return st;
 }
 
@@ -329,7 +344,7 @@ tclbm_status build_batch_graph(tclbm_batch* B) {
     cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
     tclbm_status ls = TCLBM_OK;
     if (e == cudaSuccess) {
-        ls = launch_chain(B, 2 * kGraphPairs, 0, cs);
+        ls = launch_chain(B, 2 * kGraphPairs, 0, cs, nullptr);
         e = cudaStreamEndCapture(cs, &g);
     }
     if (ls != TCLBM_OK) {
@@ -361,6 +376,7 @@ tclbm_status run_steps(tclbm_batch* B, int64_t n) {
         while (n >= 2 * kGraphPairs) {
             CK(cudaGraphLaunch(B->graph, B->stream));
             B->steps += 2 * kGraphPairs;
+            for (int64_t& d : B->done) d += 2 * kGraphPairs;
             n -= 2 * kGraphPairs;
         }
     }
@@ -448,16 +464,18 @@ tclbm_status tclbm_batch_step(tclbm_batch* B, int64_t nsteps) {
         B->steps += nsteps;
         return TCLBM_OK;
     }
+    for (int64_t& d : B->done) d = 0;
     tclbm_status st = join_streams(B, false);
     if (st == TCLBM_OK) st = upload_items(B);
     if (st == TCLBM_OK) st = upload_lattices(B);
     if (st == TCLBM_OK) st = run_steps(B, nsteps);
-    if (st != TCLBM_OK) return st;
-    for (tclbm_lattice* L : B->lats) {
-        L->cur ^= (int)(nsteps & 1);
-        L->steps += nsteps;
+    for (tclbm_lattice* L : B->lats) {  // after a failure: the steps that were launched
+        const int64_t n = B->done[tma_item(B, L) ? kGroupTma : kind_of(L)];
+        L->cur ^= (int)(n & 1);
+        L->steps += n;
     }
-    return join_streams(B, true);
+    const tclbm_status js = join_streams(B, true);
+    return st == TCLBM_OK ? js : st;
 }
 
 tclbm_status tclbm_batch_set_tile(tclbm_batch* B, int32_t tx, int32_t rows, int32_t persistent) {

@@ -79,6 +79,8 @@ namespace tclbm {
 // Records a printf-style message for tclbm_last_error() and returns `st`.
 tclbm_status fail(tclbm_status st, const char* fmt, ...) __attribute__((format(printf, 2, 3)));
 tclbm_status cuda_fail(cudaError_t e, const char* what);
+// Test hook (tclbm_test_fail_launch): whether this thread's next step launch is to fail.
+bool refuse_launch();
 // TMA row descriptors of both copies of L for strips of tx columns (box tx + 2M wide).
 tclbm_status encode_row_maps(const tclbm_lattice* L, int tx, CUtensorMap out[2]);
 // Device memory through the handle's allocator hooks (cudaMalloc / cudaFree without them).

@@ -150,3 +150,53 @@ def test_resume_from_populations_equals_an_uninterrupted_run(T, name, make):
     f2, h2 = second.populations()
     second.close()
     assert np.array_equal(f2, f_ref) and np.array_equal(h2, h_ref)
+
+
+@pytest.mark.parametrize("name,nx,ny,storage", [("chained_sr", 1536, 768, "fp16"), ("tiles", 300, 250, "fp32")])
+def test_steps_before_a_failed_launch_count(T, name, nx, ny, storage):
+    # the sixth launch of a call fails: five steps are taken and counted, and the lattice goes on
+    # from there (with its draws) as one that never saw a failure
+    case, fields = W.rayleigh_benard(nx, ny, seed=31, storage=storage)
+    case = dict(case, rounding="stochastic" if storage != "fp32" else "nearest")
+    lat = T.Lattice(case, fields)
+    T.tclbm_test_fail_launch(5)
+    with pytest.raises(T.TclbmError) as err:
+        lat.step(12)
+    T.tclbm_test_fail_launch(-1)
+    assert err.value.status == T.ECUDA and lat.steps_done == 5
+    lat.step(7)
+    got = lat.populations()
+    lat.close()
+    lat = T.Lattice(case, fields)
+    for _ in range(12):
+        lat.step(1)
+    exp = lat.populations()
+    lat.close()
+    assert np.array_equal(got[0], exp[0]) and np.array_equal(got[1], exp[1])
+
+
+def test_batch_steps_before_a_failed_launch_count(T):
+    # two kernel groups: the sixth launch is the second group's third step, so the first group
+    # has taken three steps, the second and the batch two, and the batch goes on from there
+    cases = [W.rayleigh_benard(96, 40, seed=32), W.taylor_green(64, F0=1e-6, nu=0.02)]
+    lats = [T.Lattice(c, f) for c, f in cases]
+    batch = T.Batch(lats)
+    T.tclbm_test_fail_launch(5)
+    with pytest.raises(T.TclbmError) as err:
+        batch.step(9)
+    T.tclbm_test_fail_launch(-1)
+    assert err.value.status == T.ECUDA
+    assert batch.steps_done == 2 and [lat.steps_done for lat in lats] == [3, 2]
+    batch.step(3)
+    batch.step(130)
+    assert batch.steps_done == 135 and [lat.steps_done for lat in lats] == [136, 135]
+    got = [lat.populations() for lat in lats]
+    batch.close()
+    for (c, f), lat, (gf, gh), n in zip(cases, lats, got, (136, 135)):
+        lat.close()
+        ref = T.Lattice(c, f)
+        ref.set_kernel(1)
+        ref.step(n)
+        ef, eh = ref.populations()
+        ref.close()
+        assert np.array_equal(gf, ef) and (gh is None or np.array_equal(gh, eh))
