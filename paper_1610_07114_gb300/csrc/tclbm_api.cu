@@ -750,7 +750,14 @@ tclbm_status resident_steps(tclbm_lattice* L, int64_t n, int64_t& done) {
     if (capturing(L->stream)) return TCLBM_OK;
     if (!L->board) {
         L->board_bytes = 2 * (size_t)L->prm.nx * L->prm.ny * (size_t)(L->nplanes / 3) * 16;
-        L->board = dev_alloc(L, L->board_bytes);
+        {
+            // cudaMalloc would break a global-mode capture of another stream that is open just
+            // now; this allocation is no part of one (this stream is not capturing)
+            cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+            CK(cudaThreadExchangeStreamCaptureMode(&mode));
+            L->board = dev_alloc(L, L->board_bytes);
+            CK(cudaThreadExchangeStreamCaptureMode(&mode));
+        }
         if (!L->board) {
             L->res_state = -1;
             return TCLBM_OK;

@@ -860,3 +860,31 @@ def test_lattices_on_several_streams_share_the_device(T):
     a.close()
     for f, h in got:
         assert np.array_equal(f, got[0][0]) and np.array_equal(h, got[0][1])
+
+
+def test_first_resident_run_beside_an_open_capture(T):
+    # the exchange board is allocated by the first run of 8 or more steps, here while another
+    # stream is being captured in global mode: the capture stays whole, and so does the run
+    import torch
+
+    case, fields = W.rayleigh_benard(64, 32, seed=22)
+    own, other = torch.cuda.Stream(), torch.cuda.Stream()
+    lat = T.Lattice(case, fields, stream=own.cuda_stream, memory="cuda")
+    assert "tclbm_resident" in lat.describe()
+    x = torch.zeros(64, device="cuda")
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=other, capture_error_mode="global"):
+        x.add_(1.0)
+        lat.step(20)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert float(x.sum()) == 64.0
+    got = lat.populations()
+    lat.close()
+    lat = T.Lattice(case, fields)
+    lat.set_kernel(2)
+    lat.step(20)
+    exp = lat.populations()
+    lat.close()
+    assert np.array_equal(got[0], exp[0]) and np.array_equal(got[1], exp[1])
