@@ -125,7 +125,9 @@ constexpr int kResMinNodes = 96;
 inline bool res_plan(const DevParams& p, int kind, int sms, ResPlan& best) {
     const int R = kind == RES_CORR ? 2 : 1;
     const long long N = (long long)p.nx * p.ny;
-    const int most_cells = kind == RES_ATHERMAL ? ResShape<RES_ATHERMAL, true>::CELLS : ResShape<RES_CORR, true>::CELLS;
+    const int most_cells = kind == RES_ATHERMAL  ? ResShape<RES_ATHERMAL, true>::CELLS
+                           : kind == RES_THERMAL ? ResShape<RES_THERMAL, true>::CELLS
+                                                 : ResShape<RES_CORR, false>::CELLS;
     if (N > (long long)most_cells * sms) return false;
     long long most = N / kResMinNodes;
     most = most < 1 ? 1 : (most > sms ? sms : most);

@@ -52,8 +52,10 @@ struct ResPlan {
 // 256 x 128 with 122,000 words 3.62 / 2.80.
 constexpr long long kResQuietWords = 40000;
 
+// (With the correction term tiles of more nodes than threads lose, see above.)
 template <int KIND, bool MULTI>
 struct ResShape {
+    static_assert(KIND != RES_CORR || !MULTI, "one node per thread with the correction term");
     static constexpr int R = KIND == RES_CORR ? 2 : 1;           // halo cells on each side
     static constexpr int NP = KIND == RES_ATHERMAL ? 9 : 18;     // populations per node
     static constexpr int CELLS = !MULTI ? 640 : (KIND == RES_ATHERMAL ? 2944 : 1472);  // cells of a frame
@@ -141,8 +143,8 @@ struct ResNode {
     int one_x, one_y;  // one-sided derivative: +1 at the lower wall, -1 at the upper, 0 none
 };
 
-// n >= 2 steps of the lattice from `src` to `dst`, which may be the same copy.  MULTI: more nodes than threads; a node is
-// then pulled once for its moments and again for its collision.
+// n >= 2 steps of the lattice from `src` to `dst`, which may be the same copy.  MULTI: more
+// nodes than threads.
 template <class ST, int KIND, bool MULTI, bool FAST>
 __global__ void __launch_bounds__(512, 1) tclbm_resident(const __grid_constant__ DevParams p, const ST* src,
                                                          ST* dst, uint4* __restrict__ board, int gx, int gy,
@@ -391,14 +393,6 @@ __global__ void __launch_bounds__(512, 1) tclbm_resident(const __grid_constant__
             if (mine) update(s, fw, nd, f, h, m);
         } else {
             ResNode d;
-            if (CORR) {
-                for (int t = tid; t < tasks; t += T) {
-                    if (!node_of(t, d)) continue;
-                    m = moments(fr, d, f, h);
-                    publish_phi(d, t < own, m);
-                }
-                __syncthreads();
-            }
             for (int t = tid; t < own; t += T) {
                 node_of(t, d);
                 m = moments(fr, d, f, h);
