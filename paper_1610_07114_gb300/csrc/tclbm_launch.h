@@ -121,6 +121,15 @@ inline int resident_per_sm(int storage, int kind, const ResPlan& plan, const Dev
 
 // Tiles of a resident run on `sms` CTAs (false: the lattice does not fit).  A CTA takes at
 // least kResMinNodes nodes: below that a step is all latency and more CTAs only add halo.
+// Among the shapes left the cost counts the nodes a CTA updates (in two or more turns where
+// there are more than threads), the nodes it updates for their neighbours' derivatives, and the
+// cells it reads from the board, those of columns at three times those of rows (a row's words
+// lie side by side); a tile that wraps onto itself also stores images of its edge.  Without the
+// last three, lattices without the correction term got one-row tiles: 96 x 96 thermal 5.06 us a
+// step against 2.69 with one launch per step, now 2.05; 380 x 380 5.61 / 4.97, now 4.54; 40 x 297
+// 4.73 / 3.41, now 2.20; athermal 96 x 96 2.85 / 2.39, now 1.58.  In two turns of at most 384
+// nodes no thread idles: thermal 320 x 320 4.25 us with 512 threads, 4.00 with 352 (above that
+// 512 are faster: athermal 350 x 350 3.14 / 3.22).
 constexpr int kResMinNodes = 96;
 inline bool res_plan(const DevParams& p, int kind, int sms, ResPlan& best) {
     const int R = kind == RES_CORR ? 2 : 1;
@@ -131,6 +140,7 @@ inline bool res_plan(const DevParams& p, int kind, int sms, ResPlan& best) {
     if (N > (long long)most_cells * sms) return false;
     long long most = N / kResMinNodes;
     most = most < 1 ? 1 : (most > sms ? sms : most);
+    if (most == 1 && N > 128) most = 2;  // (59 x 3: one tile 2.5 us a step, one launch per step 2.2)
     double least = 1e30;
     for (int gx = 1; gx <= most && gx <= p.nx; ++gx) {
         long long gy = most / gx;
@@ -146,10 +156,13 @@ inline bool res_plan(const DevParams& p, int kind, int sms, ResPlan& best) {
         if (cells - own > 512 || cells > most_cells) continue;
         const bool multi = own + halo > 512 || cells > 640;
         if (multi && kind == RES_CORR) continue;  // one launch per step of 2-D tiles is faster there (512 x 256: 5.9 against 7.1 us)
-        const double cost = (multi ? 1.3 : 1.0) * own + 0.4 * halo;
+        // cells read from the board: columns beside the tile (and its corners), rows above and below
+        const int cols = selfx ? 0 : 2 * R * (bh + 2 * R), rows = selfy ? 0 : 2 * R * bw;
+        const double cost = (multi ? 1.3 : 1.0) * (selfx || selfy ? 1.03 : 1.0) * own + 0.4 * halo + 0.15 * cols + 0.05 * rows;
         if (cost < least) {
             least = cost;
-            const int threads = multi ? 512 : (own + halo + 31) / 32 * 32;
+            int threads = (own + halo + 31) / 32 * 32;
+            if (multi) threads = own > 512 && own <= 768 ? (own + 63) / 64 * 32 : 512;
             best = ResPlan{gx, (int)gy, threads, multi};
         }
     }

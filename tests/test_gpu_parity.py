@@ -888,3 +888,29 @@ def test_first_resident_run_beside_an_open_capture(T):
     exp = lat.populations()
     lat.close()
     assert np.array_equal(got[0], exp[0]) and np.array_equal(got[1], exp[1])
+
+
+@pytest.mark.parametrize("nx,ny,correction", [(96, 96, False), (99, 100, False), (40, 297, False), (380, 380, False),
+                                              (320, 320, False), (59, 3, True), (96, 96, True)])
+def test_tiles_of_resident_runs_are_compact(T, nx, ny, correction):
+    # the tiles of a resident launch trade few nodes more for far fewer cells to exchange: none
+    # much longer than it is thick unless the lattice is; same states as one launch per step
+    import re
+
+    case, fields = W.random_periodic(nx, ny, seed=23, correction=correction)
+    states = []
+    for resident in (True, False):
+        lat = T.Lattice(case, fields)
+        desc = lat.describe()
+        if resident:
+            gx, gy = map(int, re.search(r"tclbm_resident grid \((\d+), (\d+)\)", desc).groups())
+            bw, bh = -(-nx // gx), -(-ny // gy)
+            assert max(bw, bh) <= max(12 * min(bw, bh), 10 * max(nx, ny) / min(nx, ny)), (bw, bh)
+            assert gx * gy > 1 and bw * bh <= 1100
+        else:
+            lat.set_kernel(2 if desc.startswith("tclbm_step_tile") else 1)
+        lat.step(21)
+        states.append(lat.populations())
+        lat.close()
+    (fa, ha), (fb, hb) = states
+    assert np.array_equal(fa, fb) and np.array_equal(ha, hb)
