@@ -151,7 +151,8 @@ tclbm_status tclbm_init_fields(tclbm_lattice* lat, const double* rho, const doub
  *
  * A lattice small enough for the shared memory of the device (about 60,000 nodes with the
  * correction term, 190,000 without, 390,000 athermal; no work term) whose kernel and
- * launch shape are the library's choice takes 8 or more steps in cooperative launches that
+ * launch shape are the library's choice takes 8 or more steps (12 or more where 2-D tiles are
+ * its one-step kernel) in cooperative launches that
  * keep its state resident (up to 1024 steps each), unless the stream is capturing.  Such a
  * launch keeps the multiprocessors it uses to itself, so where handles of this process are on
  * more than one stream of the device only lattices that fit on it eight times over (2000

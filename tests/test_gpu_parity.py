@@ -914,3 +914,24 @@ def test_tiles_of_resident_runs_are_compact(T, nx, ny, correction):
         lat.close()
     (fa, ha), (fb, hb) = states
     assert np.array_equal(fa, fb) and np.array_equal(ha, hb)
+
+
+@pytest.mark.parametrize("make,fewest", [
+    (lambda: W.rayleigh_benard(256, 128, seed=24), 12),
+    (lambda: W.random_periodic(64, 33, seed=25, correction=False), 8),
+    (lambda: W.rayleigh_benard(64, 33, seed=26), 8),  # (33 rows: no 2-D tiles)
+], ids=["tiles", "thermal", "direct"])
+def test_calls_too_short_for_a_resident_run_take_launches(T, make, fewest):
+    # filling the shared memory pays from 8 steps on, against 2-D tiles from 12; states the same
+    # on both sides of the line
+    case, fields = make()
+    states = []
+    for calls in ([fewest - 1] * 3, [3 * (fewest - 1)], [1] * (3 * (fewest - 1))):
+        lat = T.Lattice(case, fields)
+        assert f"; {fewest} steps or more: tclbm_resident" in lat.describe()
+        for n in calls:
+            lat.step(n)
+        states.append(lat.populations())
+        lat.close()
+    for f, h in states[1:]:
+        assert np.array_equal(f, states[0][0]) and np.array_equal(h, states[0][1])
