@@ -287,7 +287,8 @@ tclbm_status tclbm_set_tile(tclbm_lattice* lat, int32_t tx, int32_t ty);
  * axis nx % BX != 1 and on a walled y axis ny % BY != 1, else TCLBM_EUNSUPPORTED).  The
  * library picks per lattice size: 0 above 2,097,152 nodes, and from 1,048,576 for thermal
  * lattices with the correction term, 512 or more columns, no work term and launches that
- * chain; else 2 (or 1 where 2 does not apply).  Interior nodes evolve bit-identically under all variants; wall
+ * chain (up to 1,572,864 nodes, or up to 2,097,152 with a narrow last strip, calls of fewer
+ * than 4 steps and captured calls run under 2 all the same); else 2 (or 1 where 2 does not apply).  Interior nodes evolve bit-identically under all variants; wall
  * nodes may differ in the last bit (multiply-add contraction).  Changing the variant
  * resets the launch shape to that variant's default.  EINVAL for other values. */
 tclbm_status tclbm_set_kernel(tclbm_lattice* lat, int32_t kind);

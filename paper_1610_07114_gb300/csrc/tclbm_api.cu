@@ -661,20 +661,43 @@ bool capturing(cudaStream_t s) {
     return cap != cudaStreamCaptureStatusNone;
 }
 
+// Launches that do not chain (a call of fewer than kChainSteps steps, a stream being captured)
+// of a lattice the library gave to the TMA kernel for its chains: 2-D tiles where these are
+// the faster single steps, i.e. below 1.5 M nodes and where the last strip leaves more than a
+// tenth of the strips empty.  Measured (us per step in calls of one step, TMA / tiles):
+// 1024 x 1024 FP32 51.7 / 43.0, FP16 46.9 / 46.3; 1200 x 1000 FP32 56.8 / 49.6; 515 x 4000
+// 94.0 / 84.9; but 1448 x 1448 80.1 / 82.8, 2048 x 1024 77.5 / 81.5.  In calls of two steps
+// 1411 x 801 takes 52.5 / 47.3, of four 46 / 47.  The states are the same bit for bit.
+constexpr int64_t kChainSteps = 4;
+bool tiles_unchained(const tclbm_lattice* L) {
+    const tclbm_params& p = L->prm;
+    const long long nodes = (long long)p.nx * p.ny, strips = (p.nx + L->tx - 1) / L->tx;
+    if (!L->auto_kernel || L->kernel != KERNEL_TMA || nodes > kSmallNodes || p.work || !tile_fits(p, kTileBX, kTileBY))
+        return false;
+    return nodes < 3 * (kSmallNodes / 4) || 10LL * p.nx < 9LL * strips * L->tx;
+}
+
 tclbm_status launch_steps(tclbm_lattice* L, int64_t n) {
-    if (n > 0 && L->kernel == KERNEL_TMA) {
+    const bool chains = n > 1 && chainable(L) && !capturing(L->stream);
+    const bool tiles = (n < kChainSteps || !chains) && tiles_unchained(L);
+    if (n > 0 && L->kernel == KERNEL_TMA && !tiles) {
         tclbm_status st = ensure_maps(L);
         if (st != TCLBM_OK) return st;
     }
     // TMA launches with the correction term publish per-item completion tickets; after the
     // first launch of this run the next one waits for each item's neighbours only
-    const bool tickets = L->kernel == KERNEL_TMA && L->prm.thermal && L->prm.correction;
-    const bool chain = n > 1 && chainable(L) && !capturing(L->stream);
+    const bool tickets = L->kernel == KERNEL_TMA && L->prm.thermal && L->prm.correction && !tiles;
+    const bool chain = chains && !tiles;
     const int first = L->cur;
     tclbm_status st = TCLBM_OK;
     int64_t s = 0;
     for (; s < n; ++s) {
         StepLaunch k = step_launch(L, L->cur);
+        if (tiles) {
+            k.kernel = KERNEL_TILE;
+            k.tx = kTileBX;
+            k.ty = kTileBY;
+        }
         if (tickets) {
             k.seg_done = L->seg_done;
             k.seg_cap = (long long)(L->seg_bytes / sizeof(unsigned));
@@ -1135,6 +1158,11 @@ const char* tclbm_describe(const tclbm_lattice* L) {
         const size_t n = strlen(M->desc);
         snprintf(M->desc + n, sizeof M->desc - n, "; %d steps or more: tclbm_resident grid (%d, %d) block (%d)",
                  (int)res_min_steps(L), L->res_plan.gx, L->res_plan.gy, L->res_plan.threads);
+    }
+    if (tiles_unchained(M)) {
+        const size_t n = strlen(M->desc);
+        snprintf(M->desc + n, sizeof M->desc - n, "; fewer than %d steps: tclbm_step_tile<%d,%d>", (int)kChainSteps, kTileBX,
+                 kTileBY);
     }
     return L->desc;
 }

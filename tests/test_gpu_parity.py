@@ -613,6 +613,10 @@ def test_instances_without_options_equal_the_general_ones(T, nx, ny, walls, kern
     assert np.array_equal(fa, fb) and np.array_equal(ha, hb)
 
 
+def _with(case_fields, **kw):
+    return dict(case_fields[0], **kw), case_fields[1]
+
+
 def _tg(n, **kw):
     return W.taylor_green(n, F0=1e-6, nu=0.02, **kw)
 
@@ -933,5 +937,34 @@ def test_calls_too_short_for_a_resident_run_take_launches(T, make, fewest):
             lat.step(n)
         states.append(lat.populations())
         lat.close()
+    for f, h in states[1:]:
+        assert np.array_equal(f, states[0][0]) and np.array_equal(h, states[0][1])
+
+
+@pytest.mark.parametrize("name,make", [
+    ("rb_fp16_sr", lambda: W.rayleigh_benard(1024, 1024, seed=27, storage="fp16")),
+    ("ywalls_mu_T", lambda: _with(W.with_walls(*W.random_periodic(1100, 1000, seed=28), axis="y", kind="zouhe"),
+                                  visc_law="mu_T")),
+    ("narrow_last_strip", lambda: W.random_periodic(515, 3001, seed=29, force="taylor_green")),
+    ("xwalls_equal_rates", lambda: _with(W.with_walls(*W.random_periodic(1030, 1020, seed=30), axis="x", kind="nee"),
+                                         w_equal=True)),
+], ids=["rb_fp16_sr", "ywalls_mu_T", "narrow_last_strip", "xwalls_equal_rates"])
+def test_short_calls_on_tiles_equal_chained_ones(T, name, make):
+    # from 2^20 nodes chains of TMA launches are the faster ones, single launches only from 1.5
+    # million on: calls of one to three steps run on 2-D tiles, bit for bit the same
+    case, fields = make()
+    case = dict(case, rounding="stochastic" if case.get("storage", "fp32") != "fp32" else "nearest")
+    states = []
+    for calls in ([24], [1, 3, 2, 5, 1, 4, 3, 5], [2] * 12):
+        lat = T.Lattice(case, fields)
+        desc = lat.describe()
+        assert desc.startswith("tclbm_step_tma_corr") and "fewer than 4 steps: tclbm_step_tile" in desc, desc
+        for n in calls:
+            lat.step(n)
+        states.append(lat.populations())
+        lat.close()
+    lat = T.Lattice(*W.rayleigh_benard(2048, 1024))
+    assert "tclbm_step_tile" not in lat.describe()
+    lat.close()
     for f, h in states[1:]:
         assert np.array_equal(f, states[0][0]) and np.array_equal(h, states[0][1])
