@@ -169,7 +169,7 @@ size_t elem_of(int storage) { return storage == TCLBM_STORE_FP32 ? 4 : 2; }
 
 void derive(tclbm_lattice* L) {
     const tclbm_params& p = L->prm;
-    DevParams& d = L->dp;
+    FieldParams& d = L->dp;
     memset(&d, 0, sizeof d);
     d.skip_row = -1;  // the timeout test hook is off
     d.nx = p.nx;
@@ -325,7 +325,7 @@ __device__ __forceinline__ int wrapi(int i, int n) {
 // next step reads it: buffer_q(x - e_q) = value_q(x).  Bound by the FP64 pipe: the values
 // are formed with as few of its instructions as give the same rounding.
 template <class ST>
-__global__ void init_kernel(const DevParams p, const double* __restrict__ rho, const double* __restrict__ ux,
+__global__ void init_kernel(const FieldParams p, const double* __restrict__ rho, const double* __restrict__ ux,
                             const double* __restrict__ uy, const double* __restrict__ T, ST* __restrict__ dst,
                             int thermal, double R, double T0, double b, int force_kind, double ax, double ay,
                             double famp) {
@@ -417,7 +417,7 @@ __global__ void init_kernel(const DevParams p, const double* __restrict__ rho, c
 
 // Arbitrary populations (double [9][ny][nx] each) written in the pull layout.
 template <class ST>
-__global__ void set_pops_kernel(const DevParams p, const double* __restrict__ f, const double* __restrict__ h,
+__global__ void set_pops_kernel(const FieldParams p, const double* __restrict__ f, const double* __restrict__ h,
                                 ST* __restrict__ dst, int thermal) {
     const long long n = (long long)p.nx * p.ny;
     const int ex[9] = {0, 1, 0, -1, 0, 1, -1, -1, 1}, ey[9] = {0, 0, 1, 0, -1, 1, 1, -1, -1};
@@ -439,7 +439,7 @@ __global__ void set_pops_kernel(const DevParams p, const double* __restrict__ f,
 
 // Observable state: streamed populations with wall schemes applied (double [9][ny][nx]).
 template <bool THERMAL, class ST>
-__global__ void get_pops_kernel(const DevParams p, const ST* __restrict__ src, double* __restrict__ f,
+__global__ void get_pops_kernel(const FieldParams p, const ST* __restrict__ src, double* __restrict__ f,
                                 double* __restrict__ h) {
     const long long n = (long long)p.nx * p.ny;
     NodeWalk w(blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x, p.nx);
@@ -458,7 +458,7 @@ __global__ void get_pops_kernel(const DevParams p, const ST* __restrict__ src, d
 
 // Eq. 20 and the temperature of Section IV in FP64 from the observable state.
 template <bool THERMAL, class ST>
-__global__ void moments_kernel(const DevParams p, const ST* __restrict__ src, double* __restrict__ rho,
+__global__ void moments_kernel(const FieldParams p, const ST* __restrict__ src, double* __restrict__ rho,
                                double* __restrict__ ux, double* __restrict__ uy, double* __restrict__ T) {
     const long long n = (long long)p.nx * p.ny;
     NodeWalk w(blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x, p.nx);
@@ -484,7 +484,7 @@ __device__ __forceinline__ double warp_sum(double v) {
 
 // FP64 sums (see tclbm_diagnostics) -> one partial per block, summed by diag_finish.
 template <bool THERMAL, class ST>
-__global__ void __launch_bounds__(kDiagBlock) diag_kernel(const DevParams p, const ST* __restrict__ src,
+__global__ void __launch_bounds__(kDiagBlock) diag_kernel(const FieldParams p, const ST* __restrict__ src,
                                                           const float* __restrict__ usnap, double T_ref,
                                                           double* __restrict__ partial) {
     __shared__ double red[kDiagBlock / 32][TCLBM_NDIAG];
@@ -569,7 +569,7 @@ __global__ void diag_finish(const double* __restrict__ partial, int nblocks, con
 }
 
 template <bool THERMAL, class ST>
-__global__ void snapshot_kernel(const DevParams p, const ST* __restrict__ src, float* __restrict__ usnap) {
+__global__ void snapshot_kernel(const FieldParams p, const ST* __restrict__ src, float* __restrict__ usnap) {
     const long long n = (long long)p.nx * p.ny;
     NodeWalk w(blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x, p.nx);
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;

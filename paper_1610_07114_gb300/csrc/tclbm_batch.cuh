@@ -41,6 +41,7 @@ __global__ void __launch_bounds__(TX, 512 / TX) tclbm_step_batch(const BatchLatt
     __shared__ DevParams sp;
     __shared__ float ring[3][TX + 4];
     constexpr int kWords = (int)(sizeof(DevParams) / sizeof(int));
+    static_assert(kWords <= 4 * 32, "four loads a thread of the narrowest strips");
     constexpr int kParityWord = (int)(offsetof(DevParams, parity) / sizeof(int));
     for (int i = blockIdx.x; i < nitems; i += gridDim.x) {
         const BatchItem it = items[i];

@@ -28,7 +28,10 @@ enum { THERM_FIXED_T = 0, THERM_ADIABATIC = 1 };
 enum { VISC_NU = 0, VISC_MU = 1, VISC_MU_PROP_T = 2, VISC_W1 = 3 };
 enum { FORCE_NONE = 0, FORCE_ACCEL = 1, FORCE_TAYLOR_GREEN = 2 };
 
-// Device-side constants of one lattice (derived on the host from tclbm_params).
+// Device-side constants of one lattice (derived on the host from tclbm_params).  The batched
+// kernels copy them to shared memory for every work item: constants that the step kernels do
+// not read have no place here (168 bytes of them: a batch of one 256 x 128 lattice 9.21 us a
+// step against 8.93, of 24 up to 512 x 256 79.4 / 77.9).
 struct DevParams {
     int nx, ny, pitch;
     long long plane;  // ny * pitch elements
@@ -59,10 +62,6 @@ struct DevParams {
     unsigned ctr_add;          // steps since the counter was written (chained launches leave it alone)
     int ctr_hold;              // 1: this launch does not advance the counter
     int skip_row;              // test hook: the TMA producer never copies this source row (-1: off)
-    // FP64 constants of the field conversions (moments, diagnostics): T = inv_bR2 (E - u^2/2)
-    // with inv_bR2 = 2 / (b R), and T0, as the FP64 initialisation uses them
-    double inv_bR2, T0d;
-    double fbase_d[9], hbase_d[9], hrest;  // the rest-state populations and sum hbase
     int work;  // 1: the body force's power F.u is a source of total energy (rho E = sum h_bar + F.u/2)
 };
 

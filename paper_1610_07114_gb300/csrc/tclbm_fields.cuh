@@ -44,6 +44,14 @@ struct NodeWalk {
     }
 };
 
+// A lattice's constants with those of the field conversions in FP64: T = inv_bR2 (E - u^2/2)
+// with inv_bR2 = 2 / (b R), and T0, as the FP64 initialisation uses them; the rest-state
+// populations and sum hbase.
+struct FieldParams : DevParams {
+    double inv_bR2, T0d;
+    double fbase_d[9], hbase_d[9], hrest;
+};
+
 // (double)v without the FP64 pipe for zeros and normal numbers.
 __device__ __forceinline__ double f2d(float v) {
     const unsigned u = __float_as_uint(v), m = u & 0x7fffffffu;
@@ -150,7 +158,7 @@ struct NodeTotals {
     double rho, jx, jy, sh;
 };
 template <bool THERMAL>
-__device__ __forceinline__ NodeTotals node_totals(const DevParams& p, const NodeSums& s, const float (&f)[9],
+__device__ __forceinline__ NodeTotals node_totals(const FieldParams& p, const NodeSums& s, const float (&f)[9],
                                                   const float (&h)[9]) {
     if (s.narrow())
         return NodeTotals{sum_value(1.0, s.drho), sum_value(s.jx), sum_value(s.jy), THERMAL ? sum_value(p.hrest, s.sdh) : 0.0};
@@ -191,7 +199,7 @@ __device__ __forceinline__ NodeFields node_velocity(const DevParams& p, const No
 
 // Temperature of Section IV; hrest: the rest value of sum h_bar, uu = |u|^2.
 template <bool THERMAL>
-__device__ __forceinline__ double node_temperature(const DevParams& p, const NodeFields& n, double sh, double uu, int x,
+__device__ __forceinline__ double node_temperature(const FieldParams& p, const NodeFields& n, double sh, double uu, int x,
                                                    int y) {
     if (!THERMAL) return p.T0d;
     if (p.work) {  // rho E = sum h_bar + F.u / 2

@@ -8,6 +8,7 @@
 
 #include "tclbm.h"
 #include "tclbm_device.cuh"
+#include "tclbm_fields.cuh"
 #include "tclbm_launch.h"
 
 namespace tclbm {
@@ -26,7 +27,7 @@ using tclbm::KERNEL_TMA;
 
 struct tclbm_lattice {
     tclbm_params prm;
-    DevParams dp;
+    tclbm::FieldParams dp;
     cudaStream_t stream = nullptr;
     tclbm_alloc_fn alloc = nullptr;
     tclbm_free_fn free_fn = nullptr;
