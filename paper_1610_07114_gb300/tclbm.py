@@ -406,6 +406,8 @@ class Lattice:
                 a = a.contiguous().double()
             else:
                 a = np.ascontiguousarray(a, dtype=np.float64)
+                if a.size == 1:  # one value everywhere (athermal cases give T so)
+                    a = np.full((self.ny, self.nx), a.flat[0])
             arrs.append(a)
         self._keep = arrs
         tclbm_init_fields(self.handle, *[_ptr(a) for a in arrs], on_dev)

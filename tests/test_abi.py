@@ -120,3 +120,20 @@ def test_pages_of_host_outputs_are_made_present_without_a_write(T):
     # what the host may not write is left to the copy to refuse
     ro = mmap.mmap(-1, 2 * mmap.PAGESIZE, prot=mmap.PROT_READ)
     T.tclbm_test_populate(np.frombuffer(ro, dtype=np.uint8).ctypes.data, 2 * mmap.PAGESIZE)
+
+
+def test_a_field_given_as_one_value_is_handed_over_for_every_node(T, monkeypatch):
+    # the library reads ny * nx values of each host field, so one number (athermal cases give T as
+    # one) has to become an array of that size
+    import numpy as np
+
+    from paper_1610_07114_gb300 import workloads as W
+
+    case, fields = W.random_periodic(40, 24, seed=3, thermal=False)
+    assert np.ndim(fields["T"]) == 0
+    lat = object.__new__(T.Lattice)
+    lat.handle, lat.nx, lat.ny = None, 40, 24
+    monkeypatch.setattr(T, "tclbm_init_fields", lambda *a: None)
+    lat.init_fields(fields)
+    assert [a.size for a in lat._keep] == [40 * 24] * 4
+    assert np.array_equal(lat._keep[3].ravel(), np.full(40 * 24, fields["T"])) and lat._keep[0] is fields["rho"]
