@@ -241,6 +241,11 @@ const char* tclbm_describe(const tclbm_lattice* lat);
  * it).  row = -1 turns the hook off.  EINVAL for other rows. */
 tclbm_status tclbm_test_skip_row(tclbm_lattice* lat, int32_t row);
 
+/* Test hook for resident runs (no counterpart in the paper): the next run numbers its states
+ * from `number` on (they start over, on a cleared exchange board, where 32 bits end).  EINVAL
+ * before the handle's first resident run and for numbers already used. */
+tclbm_status tclbm_test_run_number(tclbm_lattice* lat, uint32_t number);
+
 /* Test hook for failed launches (no counterpart in the paper): of the step launches (or
  * resident runs) that calls on this thread make from now on, the one after `after` others is
  * not made and reported as failed (TCLBM_ECUDA).  The steps launched before it are taken and

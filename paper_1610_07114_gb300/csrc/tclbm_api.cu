@@ -1078,6 +1078,13 @@ tclbm_status tclbm_test_skip_row(tclbm_lattice* L, int32_t row) {
     return TCLBM_OK;
 }
 
+tclbm_status tclbm_test_run_number(tclbm_lattice* L, uint32_t number) {
+    if (!L) return fail(TCLBM_EINVAL, "lattice is NULL");
+    if (!L->board || number < L->res_tag) return fail(TCLBM_EINVAL, "no resident run yet, or numbers would come again");
+    L->res_tag = number;
+    return TCLBM_OK;
+}
+
 tclbm_status tclbm_test_fail_launch(int64_t after) {
     if (after < -1) return fail(TCLBM_EINVAL, "after must be >= -1");
     g_refuse_in = after;

@@ -100,6 +100,8 @@ _lib.tclbm_test_skip_row.argtypes = [_vp, ctypes.c_int32]
 _lib.tclbm_test_skip_row.restype = ctypes.c_int
 _lib.tclbm_test_rcp.argtypes = [_vp, _vp, ctypes.c_int64, _vp]
 _lib.tclbm_test_rcp.restype = ctypes.c_int
+_lib.tclbm_test_run_number.argtypes = [_vp, ctypes.c_uint32]
+_lib.tclbm_test_run_number.restype = ctypes.c_int
 _lib.tclbm_test_fail_launch.argtypes = [ctypes.c_int64]
 _lib.tclbm_test_fail_launch.restype = ctypes.c_int
 _lib.tclbm_test_div.argtypes = [_vp, _vp, _vp, ctypes.c_int64, _vp]
@@ -219,6 +221,10 @@ def tclbm_test_skip_row(h, row):
 
 def tclbm_test_rcp(x, y, n, stream=None):
     _check(_lib.tclbm_test_rcp(x, y, int(n), stream), "tclbm_test_rcp")
+
+
+def tclbm_test_run_number(h, number):
+    _check(_lib.tclbm_test_run_number(h, number), "tclbm_test_run_number")
 
 
 def tclbm_test_fail_launch(after):

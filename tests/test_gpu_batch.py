@@ -285,3 +285,42 @@ def test_tma_fed_batch_matches_fp64_oracle(T):
 
     e = field_errors(g, o.moments(), case)
     assert e["rho"] <= 1e-5 and e["u"] <= 1e-5 and e["T"] <= 1e-5, e
+
+
+@pytest.mark.parametrize("mode", ["global", "thread_local"])
+def test_first_call_of_several_groups_captured_and_replayed(T, mode):
+    # the side streams of the kernel groups are forked and joined inside the caller's capture, on
+    # the batch's first call too: the replays advance every lattice as calls do
+    import torch
+
+    def lattices():
+        cases = [W.rayleigh_benard(128, 40, seed=51), W.random_periodic(70, 20, seed=52, correction=False),
+                 W.taylor_green(64, F0=1e-6, nu=0.02), W.rayleigh_benard(48, 24, seed=53)]
+        return [T.Lattice(c, f, stream=stream.cuda_stream) for c, f in cases]
+
+    stream = torch.cuda.Stream()
+    lats = lattices()
+    batch = T.Batch(lats, stream=stream.cuda_stream)
+    batch.set_tma(64, 16)
+    stream.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream, capture_error_mode=mode):
+        batch.step(4)
+    for _ in range(3):
+        with torch.cuda.stream(stream):
+            graph.replay()
+    stream.synchronize()
+    got = [lat.populations() for lat in lats]
+    batch.close()
+    for lat in lats:
+        lat.close()
+    refs = lattices()
+    batch = T.Batch(refs, stream=stream.cuda_stream)
+    batch.set_tma(64, 16)
+    batch.step(12)
+    for (f, h), ref in zip(got, refs):
+        ef, eh = ref.populations()
+        assert np.array_equal(f, ef) and (h is None or np.array_equal(h, eh))
+    batch.close()
+    for ref in refs:
+        ref.close()

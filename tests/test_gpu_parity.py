@@ -968,3 +968,128 @@ def test_short_calls_on_tiles_equal_chained_ones(T, name, make):
     lat.close()
     for f, h in states[1:]:
         assert np.array_equal(f, states[0][0]) and np.array_equal(h, states[0][1])
+
+
+def _walls(cf, axis, kind, therm="fixed", **kw):
+    case, fields = W.with_walls(*cf, axis=axis, kind=kind)
+    for side in (axis + "-", axis + "+"):
+        case["walls"][side] = dict(case["walls"][side], therm=therm)
+    return dict(case, **kw), fields
+
+
+GENERAL_CASES = [
+    # options that the instances without them do not know: laws, equal rates, a force in space
+    ("mu_ywalls", lambda: _walls(W.random_periodic(97, 66, seed=101), "y", "zouhe", visc_law="mu")),
+    ("mu_T_xwalls", lambda: _walls(W.random_periodic(100, 51, seed=102), "x", "nee", "adiabatic", visc_law="mu_T")),
+    ("w1_periodic", lambda: _with(W.random_periodic(131, 7, seed=103), visc_law="w1", visc=1.1)),
+    ("equal_rates_ywalls", lambda: _walls(W.random_periodic(60, 61, seed=104), "y", "equilibrium", w_equal=True)),
+    ("taylor_green_force", lambda: W.random_periodic(90, 70, seed=105, force="taylor_green")),
+    # walls without the correction term: one node per thread, and more nodes than threads
+    ("thermal_ywalls", lambda: _walls(W.random_periodic(150, 90, seed=106, correction=False), "y", "zouhe", "adiabatic")),
+    ("thermal_xwalls_many", lambda: _walls(W.random_periodic(301, 333, seed=107, correction=False), "x", "nee")),
+    ("thermal_ywalls_many", lambda: _walls(W.random_periodic(401, 301, seed=108, correction=False), "y", "zouhe",
+                                           visc_law="mu_T")),
+    ("athermal_xwalls", lambda: _walls(W.random_periodic(120, 77, seed=109, thermal=False), "x", "zouhe")),
+    ("athermal_ywalls_many", lambda: _walls(W.random_periodic(411, 390, seed=110, thermal=False), "y", "nee", w_equal=True)),
+    ("athermal_xwalls_many", lambda: _walls(W.random_periodic(505, 600, seed=111, thermal=False), "x", "equilibrium")),
+]
+
+
+@pytest.mark.parametrize("storage,rounding", [("fp32", "nearest"), ("fp16", "stochastic")])
+@pytest.mark.parametrize("name,make", GENERAL_CASES, ids=[c[0] for c in GENERAL_CASES])
+def test_resident_runs_of_every_option_equal_one_launch_per_step(T, name, make, storage, rounding):
+    case, fields = make()
+    case = dict(case, storage=storage, rounding=rounding)
+    states = []
+    for resident in (True, False):
+        lat = T.Lattice(case, fields)
+        desc = lat.describe()
+        assert "tclbm_resident" in desc, desc
+        if not resident:
+            lat.set_kernel(2 if desc.startswith("tclbm_step_tile") else 1)
+        for n in (13, 1, 24):
+            lat.step(n)
+        assert np.isfinite(lat.diagnostics()).all()
+        states.append(lat.populations())
+        lat.close()
+    (fa, ha), (fb, hb) = states
+    assert np.array_equal(fa, fb)
+    assert not case["thermal"] or np.array_equal(ha, hb)
+
+
+@pytest.mark.parametrize("make", [lambda: W.rayleigh_benard(96, 48, seed=33, storage="fp16"), lambda: W.couette(8, 64),
+                                  lambda: _tg(64, storage="bf16")], ids=["rb_fp16_sr", "couette", "athermal_bf16_sr"])
+def test_long_resident_calls_and_state_numbers_that_start_over(T, make):
+    # one call of several launches (1024 steps each at most), then runs across the end of the 32-bit
+    # state numbers, where the exchange board is cleared: against one launch per step
+    case, fields = make()
+    case = dict(case, rounding="stochastic" if case.get("storage", "fp32") != "fp32" else "nearest")
+    states = []
+    for resident in (True, False):
+        lat = T.Lattice(case, fields)
+        if not resident:
+            lat.set_kernel(2 if lat.describe().startswith("tclbm_step_tile") else 1)
+        else:
+            with pytest.raises(T.TclbmError):
+                T.tclbm_test_run_number(lat.handle, 5)
+        lat.step(2 * 1024 + 37)
+        if resident:
+            T.tclbm_test_run_number(lat.handle, 2 ** 32 - 31)
+        for n in (15, 14, 20, 17):
+            lat.step(n)
+        if resident:
+            T.tclbm_test_run_number(lat.handle, 2 ** 32 - 1 - 16)  # a run that ends on the last number
+        lat.step(16)
+        lat.step(16)
+        states.append(lat.populations())
+        lat.close()
+    (fa, ha), (fb, hb) = states
+    assert np.array_equal(fa, fb)
+    assert not case["thermal"] or np.array_equal(ha, hb)
+
+
+@pytest.mark.parametrize("storage,rounding", [("fp32", "nearest"), ("fp16", "stochastic"), ("bf16", "nearest")])
+@pytest.mark.parametrize("nx,ny,walls,kernel", [(640, 45, None, 0), (515, 40, ("y", "zouhe"), 0), (530, 32, ("x", "nee"), 0),
+                                                (96, 64, ("y", "nee"), None), (131, 50, None, None)])
+def test_instances_without_options_equal_the_general_ones_on_wide_strips_and_resident(T, nx, ny, walls, kernel, storage,
+                                                                                    rounding):
+    # as above, in the 128-wide strips that large lattices run and in the resident kernel
+    case, fields = W.random_periodic(nx, ny, seed=112, force="none", storage=storage)
+    if walls:
+        case, fields = W.with_walls(case, fields, axis=walls[0], kind=walls[1])
+    case = dict(case, rounding=rounding)
+    states = []
+    for force in ("none", "taylor_green"):
+        lat = T.Lattice(dict(case, force={"kind": force, "ax": 0.0, "ay": 0.0, "amp": 0.0}), fields)
+        if kernel is None:
+            assert "tclbm_resident" in lat.describe()
+        else:
+            lat.set_kernel(kernel)
+            assert lat.describe().startswith("tclbm_step_tma_corr<128")
+        lat.step(25)
+        states.append(lat.populations())
+        lat.close()
+    (fa, ha), (fb, hb) = states
+    assert np.array_equal(fa, fb) and np.array_equal(ha, hb)
+
+
+@pytest.mark.parametrize("name,make", GENERAL_CASES[:5], ids=[c[0] for c in GENERAL_CASES[:5]])
+def test_tma_direct_and_tile_kernels_agree_for_every_option(T, name, make):
+    # the library takes one kernel or another by size and call length: nodes at walls included,
+    # the states are the same bit for bit
+    case, fields = make()
+    states = []
+    for kernel in (0, 1, 2):
+        lat = T.Lattice(case, fields)
+        try:
+            lat.set_kernel(kernel)
+        except T.TclbmError:  # (no 2-D tiles for this size)
+            assert kernel == 2
+            lat.close()
+            continue
+        lat.step(25)
+        states.append(lat.populations())
+        lat.close()
+    assert len(states) >= 2
+    for f, h in states[1:]:
+        assert np.array_equal(f, states[0][0]) and np.array_equal(h, states[0][1])
