@@ -45,27 +45,44 @@ def _peaks():
         return 6800.0, "fallback"
 
 
+KERNEL_SOURCES = tuple(f"paper_1610_07114_gb300/csrc/{f}"
+                       for f in ("tclbm_device.cuh", "tclbm_tma.cuh", "tclbm_resident.cuh"))
+
+
 def _kernel_source_hash():
     h = hashlib.sha256()
-    # device code of the single-lattice step kernels (direct and TMA-fed)
-    for rel in ("paper_1610_07114_gb300/csrc/tclbm_device.cuh", "paper_1610_07114_gb300/csrc/tclbm_tma.cuh"):
+    # device code of the single-lattice step kernels (direct, TMA-fed, resident)
+    for rel in KERNEL_SOURCES:
         with open(os.path.join(ROOT, rel), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
 
 
-def _profiled_traffic(key):
-    """DRAM bytes per launch from a committed ncu summary, if taken on the current kernel source."""
+def _profiled_traffic(key, steps=1):
+    """DRAM bytes per launch from a committed ncu summary, if taken on the current kernel source
+    and for a launch of as many time steps (the resident kernel takes many in one)."""
     path = os.path.join(ROOT, "profiles", "traffic.json")
     try:
         with open(path) as fh:
             d = json.load(fh)
         e = d.get(key)
-        if e and e.get("source_hash") == _kernel_source_hash():
+        if e and e.get("source_hash") == _kernel_source_hash() and e.get("steps_per_launch", 1) == steps:
             return e.get("bytes_per_launch")
     except Exception:
         pass
     return None
+
+
+RESIDENT_STEPS = 1024  # steps of one resident launch at most
+
+
+def _step_launches(desc, steps):
+    """Step kernels launched by one call of `steps` steps (desc: the lattice's description)."""
+    if "tclbm_resident" not in desc:
+        return steps
+    fewest = int(desc.split(" steps or more: tclbm_resident")[0].split()[-1])
+    full, rest = divmod(steps, RESIDENT_STEPS)
+    return full + (1 if rest >= fewest else rest)
 
 
 class ClockSampler:
@@ -476,7 +493,7 @@ def bench_gpu(args):
     achieved = BYTES_PER_LU[args.storage] * n / kernel_s / 1e9
     wkey = f"rb_{args.nx}x{args.ny}_{args.storage}"
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
-                "traffic": _profiled_traffic(wkey), "peak_source": f"{peak_kind} hbm_gbs (copy)",
+                "traffic": _profiled_traffic(wkey, args.chunk if _step_launches(desc, args.chunk) == 1 else 1), "peak_source": f"{peak_kind} hbm_gbs (copy)",
                 "kernel": desc, "bytes_per_LU": BYTES_PER_LU[args.storage],
                 "note": "the 4.7 MB state stays in L2 within a chunk; see roofline_probe for lattices >> L2"}
     cpu = None
@@ -507,8 +524,7 @@ def bench_gpu(args):
         "serving": serving,
         "cpu_baseline": cpu,
         "clocks": clk,
-        # (a resident run takes up to 1024 steps in one launch)
-        "gpu_launches": args.steps * ((-(-args.chunk // 1024) if "tclbm_resident" in desc else args.chunk) + 2),
+        "gpu_launches": args.steps * (_step_launches(desc, args.chunk) + 2),
         "nusselt": nu_num,
         "kernel_us": kernel_s * 1e6,
     }
