@@ -758,11 +758,12 @@ bool resident_planned(tclbm_lattice* L) {
             coop = 0;
         }
         L->res_state = coop && res_plan(L->dp, res_kind(L->prm), sm_count(), L->res_plan) ? 1 : -1;
-        if (L->res_state > 0)
-            L->res_small = (long long)resident_per_sm(L->storage, res_kind(L->prm), L->res_plan, L->dp) * sm_count() >=
-                           kResShared * L->res_plan.gx * L->res_plan.gy;
     }
-    return L->res_state > 0 && (L->res_small || only_stream(L->use));
+    if (L->res_state < 0 || only_stream(L->use)) return L->res_state > 0;
+    if (L->res_small < 0)
+        L->res_small = (long long)resident_per_sm(L->storage, res_kind(L->prm), L->res_plan, L->dp) * sm_count() >=
+                       kResShared * L->res_plan.gx * L->res_plan.gy;
+    return L->res_small > 0;
 }
 
 // Advances L by as many of n steps as resident launches take (`done`); 0 where they do not

@@ -62,7 +62,7 @@ struct tclbm_lattice {
     // number of the last state a run has used
     bool auto_kernel = true;
     int res_state = 0;  // 0 not planned yet, 1 planned, -1 does not apply
-    bool res_small = false;  // several such runs fit on the device at once
+    int res_small = -1;  // whether several such runs fit on the device at once (-1: not asked yet)
     tclbm::StreamUse* use = nullptr;  // this handle's entry in the streams in use
     tclbm::ResPlan res_plan{};
     void* board = nullptr;
