@@ -268,9 +268,11 @@ tclbm_status tclbm_test_div(const double* a, const double* x, double* y, int64_t
 
 /* Test hook for the node order of the field conversions (no counterpart in the paper; host
  * code, no device work): x[k], y[k] = column and row, in a lattice nx wide, of node
- * first + k * stride as a thread of the conversion kernels counts them, for k < count.
+ * first + k * stride, for k < count: as a thread of the conversion kernels counts them, or
+ * (divide != 0) as the initial fields divide for them.
  * EINVAL on nx < 1, count < 0 or NULL arrays with count > 0. */
-tclbm_status tclbm_test_node_walk(uint32_t first, uint32_t stride, int32_t nx, int64_t count, int32_t* x, int32_t* y);
+tclbm_status tclbm_test_node_walk(uint32_t first, uint32_t stride, int32_t nx, int64_t count, int32_t divide, int32_t* x,
+                                  int32_t* y);
 
 /* Test hook for host outputs (no counterpart in the paper; host code, no device work): makes
  * the pages of `array` present as tclbm_moments() and tclbm_get_populations() do for

@@ -330,10 +330,10 @@ __global__ void init_kernel(const FieldParams p, const double* __restrict__ rho,
                             int thermal, double R, double T0, double b, int force_kind, double ax, double ay,
                             double famp) {
     const long long n = (long long)p.nx * p.ny;
-    NodeWalk w(blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x, p.nx);
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x, w.next(p.nx)) {
-        const int x = w.x, y = w.y;
+    const bool wide = wide_nodes(n);
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+        int x, y;
+        node_xy(i, p.nx, wide, x, y);
         const double r = rho[i], vx = ux[i], vy = uy[i], t = thermal ? T[i] : T0;
         const double RT = __dmul_rn(R, t), ux2 = __dmul_rn(vx, vx), uy2 = __dmul_rn(vy, vy);
         const double qx = __dadd_rn(RT, ux2), qy = __dadd_rn(RT, uy2);
@@ -1127,13 +1127,16 @@ tclbm_status tclbm_test_div(const double* a, const double* x, double* y, int64_t
     return TCLBM_OK;
 }
 
-tclbm_status tclbm_test_node_walk(uint32_t first, uint32_t stride, int32_t nx, int64_t count, int32_t* x, int32_t* y) {
+tclbm_status tclbm_test_node_walk(uint32_t first, uint32_t stride, int32_t nx, int64_t count, int32_t divide, int32_t* x,
+                                  int32_t* y) {
     if (nx < 1 || count < 0 || (count > 0 && (!x || !y))) return fail(TCLBM_EINVAL, "bad node walk");
     NodeWalk w(first, stride, nx);
     for (int64_t k = 0; k < count; ++k, w.next(nx)) {
         x[k] = w.x;
         y[k] = w.y;
     }
+    const bool wide = wide_nodes(first + (count > 0 ? count - 1 : 0) * (long long)stride + 1);
+    for (int64_t k = 0; divide && k < count; ++k) node_xy(first + k * (long long)stride, nx, wide, x[k], y[k]);
     return TCLBM_OK;
 }
 

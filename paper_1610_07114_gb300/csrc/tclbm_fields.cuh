@@ -44,6 +44,22 @@ struct NodeWalk {
     }
 };
 
+// The same of node i by division, for the initial fields: bound by the FP64 pipe, they lose 2.4 %
+// to the counted walk (4096 x 2048 1983 / 2030 us), where storing populations gains from it
+// (2048 x 1024 234 / 186).  `wide`: more than 2^32 nodes.
+__host__ __device__ __forceinline__ void node_xy(long long i, int nx, bool wide, int& x, int& y) {
+    if (wide) {
+        const long long r = i / nx;
+        y = (int)r;
+        x = (int)(i - r * nx);
+    } else {
+        const unsigned r = (unsigned)i / (unsigned)nx;
+        y = (int)r;
+        x = (int)((unsigned)i - r * (unsigned)nx);
+    }
+}
+__host__ __device__ __forceinline__ bool wide_nodes(long long n) { return n > (1LL << 32); }
+
 // A lattice's constants with those of the field conversions in FP64: T = inv_bR2 (E - u^2/2)
 // with inv_bR2 = 2 / (b R), and T0, as the FP64 initialisation uses them; the rest-state
 // populations and sum hbase.

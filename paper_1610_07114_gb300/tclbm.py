@@ -107,7 +107,8 @@ _lib.tclbm_test_fail_launch.restype = ctypes.c_int
 _lib.tclbm_test_div.argtypes = [_vp, _vp, _vp, ctypes.c_int64, _vp]
 _lib.tclbm_test_div.restype = ctypes.c_int
 _i32p = ctypes.POINTER(ctypes.c_int32)
-_lib.tclbm_test_node_walk.argtypes = [ctypes.c_uint32, ctypes.c_uint32, ctypes.c_int32, ctypes.c_int64, _i32p, _i32p]
+_lib.tclbm_test_node_walk.argtypes = [ctypes.c_uint32, ctypes.c_uint32, ctypes.c_int32, ctypes.c_int64, ctypes.c_int32,
+                                      _i32p, _i32p]
 _lib.tclbm_test_node_walk.restype = ctypes.c_int
 _lib.tclbm_test_populate.argtypes = [_vp, ctypes.c_size_t]
 _lib.tclbm_test_populate.restype = ctypes.c_int
@@ -235,9 +236,10 @@ def tclbm_test_div(a, x, y, n, stream=None):
     _check(_lib.tclbm_test_div(a, x, y, int(n), stream), "tclbm_test_div")
 
 
-def tclbm_test_node_walk(first, stride, nx, count):
+def tclbm_test_node_walk(first, stride, nx, count, divide=False):
     x, y = np.zeros(count, dtype=np.int32), np.zeros(count, dtype=np.int32)
-    _check(_lib.tclbm_test_node_walk(first, stride, nx, count, x.ctypes.data_as(_i32p), y.ctypes.data_as(_i32p)),
+    _check(_lib.tclbm_test_node_walk(first, stride, nx, count, int(divide), x.ctypes.data_as(_i32p),
+                                      y.ctypes.data_as(_i32p)),
            "tclbm_test_node_walk")
     return x, y
 

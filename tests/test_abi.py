@@ -137,3 +137,15 @@ def test_a_field_given_as_one_value_is_handed_over_for_every_node(T, monkeypatch
     lat.init_fields(fields)
     assert [a.size for a in lat._keep] == [40 * 24] * 4
     assert np.array_equal(lat._keep[3].ravel(), np.full(40 * 24, fields["T"])) and lat._keep[0] is fields["rho"]
+
+
+@pytest.mark.parametrize("nx", [1, 511, 65536, (1 << 20) + 7])
+@pytest.mark.parametrize("first,stride", [(0, 1 << 31), ((1 << 32) - 1, (1 << 32) - 1), (5, 622592)])
+def test_nodes_beyond_32_bits_keep_their_rows_in_initial_fields(T, nx, first, stride):
+    # the same by division: 32 bits wide only where the lattice has no node past them
+    count = 9 if nx > 1 else 1
+    x, y = T.tclbm_test_node_walk(first, stride, nx, count, divide=True)
+    for k in range(count):
+        node = first + k * stride
+        if node // nx < 1 << 31:
+            assert (int(x[k]), int(y[k])) == (node % nx, node // nx), (node, nx)
