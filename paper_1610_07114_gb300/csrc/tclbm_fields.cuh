@@ -13,10 +13,10 @@
 //   - one reciprocal of rho serves the three divisions, each corrected by its remainder.
 // The results are as near the exact ones as those of the plain FP64 expressions (compared
 // with quad precision over the flows of the performance cases).
-// Measured before / after (us): 4096 x 2048 FP32, moments 1962 / 701, diagnostics 2447 /
-// 1026, velocity snapshot 1155 / 468, initial fields 3337 / 1933 (their bytes take 129, 89,
-// 99 and 129); 2048 x 1024 populations in 258 / 187, out 236 / 113.  An FP64 instruction per
-// node costs 23 us at 4096 x 2048; about 28, 42, 19 and 84 are left.
+// Measured before / after (us): 4096 x 2048 FP32, moments 1962 / 596, diagnostics 2447 / 838,
+// velocity snapshot 1155 / 413, initial fields 3337 / 1983 (their bytes take 129, 89, 99 and
+// 129); 2048 x 1024 populations in 258 / 186, out 236 / 113.  An FP64 instruction per node
+// costs 23 us at 4096 x 2048; about 26, 36, 18 and 86 are left.
 #pragma once
 
 #include "tclbm_device.cuh"
@@ -243,7 +243,7 @@ struct Running {
     }
     __device__ __forceinline__ void add(const Sum3& p) {
         add(p.hi);
-        add(p.mid);  // (lo is below 2^-48 of a deviation and 2^-72 of the sum it would enter)
+        add(p.mid);  // (lo is below 2^-48 of this node's sum)
     }
     __device__ __forceinline__ double value() const { return (f2d(c) + f2d(b)) + f2d(a); }
 };

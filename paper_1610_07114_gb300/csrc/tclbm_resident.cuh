@@ -27,9 +27,10 @@
 //
 // What bounds it: the exchange (a store through L2 to a neighbour's read, 1 to 1.5 us) and
 // the dependent chain of one node update (about 1 us at one or two warps per scheduler).
-// Measured (GB300, us per step against one launch per step): thermal with the correction
-// term 8 x 64 2.1 / 2.7, 128 x 64 2.3 / 2.8, 4096 x 4 2.6 / 3.9, 256 x 128 2.8 / 3.1,
-// 300 x 150 3.2 / 4.3; athermal 64 x 64 1.5 / 2.5, 256 x 256 2.0 / 3.0, 512 x 512 5.9 / 8.1.
+// Measured (GB300, us per step in runs of 200 against one launch per step): thermal with the
+// correction term 8 x 64 2.1 / 2.8, 128 x 64 2.4 / 2.9, 4096 x 4 2.6 / 3.9, 256 x 128 2.94 / 3.15
+// (periodic 2.81 / 2.79), 300 x 150 3.3 / 4.2; without it 128 x 128 1.9 / 2.8, 400 x 400 5.4 / 6.1;
+// athermal 64 x 64 1.6 / 2.6, 256 x 256 2.1 / 3.1, 512 x 512 5.9 / 8.2.
 // With the correction term tiles of more nodes than threads lose (512 x 256: 7.1 / 5.9).
 //
 // The arithmetic is that of the one-step kernels, node for node.
@@ -47,9 +48,9 @@ struct ResPlan {
 };
 
 // Words all CTAs read from the board per step above which they poll with one lane per warp.
-// Measured (all lanes / one lane, us per step): 64 x 32 with 12,600 words 2.07 / 2.20, the
-// 4096 x 4 shock tube with 29,000 words 2.59 / 2.98, 128 x 64 with 48,000 words 2.45 / 2.40,
-// 256 x 128 with 122,000 words 3.62 / 2.80.
+// Measured (all lanes / one lane, us per step): 64 x 32 with 12,600 words 2.35 / 2.33, the
+// 4096 x 4 shock tube with 29,000 words 2.59 / 2.75, 128 x 64 with 48,000 words 2.53 / 2.55,
+// 256 x 128 with 122,000 words 3.49 / 2.94 (periodic 3.57 / 2.78).
 constexpr long long kResQuietWords = 40000;
 
 // (With the correction term tiles of more nodes than threads lose, see above.)
