@@ -274,11 +274,6 @@ tclbm_status tclbm_test_div(const double* a, const double* x, double* y, int64_t
 tclbm_status tclbm_test_node_walk(uint32_t first, uint32_t stride, int32_t nx, int64_t count, int32_t divide, int32_t* x,
                                   int32_t* y);
 
-/* Test hook for host outputs (no counterpart in the paper; host code, no device work): makes
- * the pages of `array` present as tclbm_moments() and tclbm_get_populations() do for
- * pageable outputs before their copies.  Changes no byte.  EINVAL on NULL. */
-tclbm_status tclbm_test_populate(void* array, size_t bytes);
-
 /* Launch-shape override for tuning; 0 keeps the library's choice.  Kernel variants 0
  * and 1: strip width tx (32, 64 or 128 nodes) and rows per CTA ty (>= 1); under variant 0,
  * where the grid spans more than two waves of resident CTAs, ty is a multiple of 16 and

@@ -110,8 +110,6 @@ _i32p = ctypes.POINTER(ctypes.c_int32)
 _lib.tclbm_test_node_walk.argtypes = [ctypes.c_uint32, ctypes.c_uint32, ctypes.c_int32, ctypes.c_int64, ctypes.c_int32,
                                       _i32p, _i32p]
 _lib.tclbm_test_node_walk.restype = ctypes.c_int
-_lib.tclbm_test_populate.argtypes = [_vp, ctypes.c_size_t]
-_lib.tclbm_test_populate.restype = ctypes.c_int
 _lib.tclbm_set_kernel.argtypes = [_vp, ctypes.c_int32]
 _lib.tclbm_set_kernel.restype = ctypes.c_int
 _lib.tclbm_copy_rows.argtypes = [_vp, ctypes.c_int32, _vp, ctypes.c_int32, ctypes.c_int32]
@@ -242,10 +240,6 @@ def tclbm_test_node_walk(first, stride, nx, count, divide=False):
                                       y.ctypes.data_as(_i32p)),
            "tclbm_test_node_walk")
     return x, y
-
-
-def tclbm_test_populate(array, nbytes):
-    _check(_lib.tclbm_test_populate(array, nbytes), "tclbm_test_populate")
 
 
 def tclbm_copy_rows(dst, dst_row, src, src_row, rows):

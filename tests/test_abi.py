@@ -96,32 +96,6 @@ def test_nodes_beyond_32_bits_keep_their_rows(T, nx, first, stride):
             assert (int(x[k]), int(y[k])) == (node % nx, node // nx), (node, nx)
 
 
-def test_pages_of_host_outputs_are_made_present_without_a_write(T):
-    # device work queued earlier may still read the array a call is about to overwrite in
-    # stream order: its bytes stay as they are, on its pages and around them
-    import mmap
-    import resource
-
-    import numpy as np
-
-    rng = np.random.default_rng(3)
-    a = rng.integers(1, 256, 50 * mmap.PAGESIZE + 123, dtype=np.uint8)
-    want = a.copy()
-    for lo, n in ((0, a.size), (1, a.size - 1), (4097, 3 * mmap.PAGESIZE), (777, 5)):
-        T.tclbm_test_populate(a.ctypes.data + lo, n)
-        assert np.array_equal(a, want)
-    # and fresh pages are there afterwards: writing all of them takes next to no fault
-    fresh = mmap.mmap(-1, 400 * mmap.PAGESIZE)
-    buf = np.frombuffer(fresh, dtype=np.uint8)
-    T.tclbm_test_populate(buf.ctypes.data, buf.size)
-    before = resource.getrusage(resource.RUSAGE_SELF).ru_minflt
-    buf[::mmap.PAGESIZE] = 1
-    assert resource.getrusage(resource.RUSAGE_SELF).ru_minflt - before < 40
-    # what the host may not write is left to the copy to refuse
-    ro = mmap.mmap(-1, 2 * mmap.PAGESIZE, prot=mmap.PROT_READ)
-    T.tclbm_test_populate(np.frombuffer(ro, dtype=np.uint8).ctypes.data, 2 * mmap.PAGESIZE)
-
-
 def test_a_field_given_as_one_value_is_handed_over_for_every_node(T, monkeypatch):
     # the library reads ny * nx values of each host field, so one number (athermal cases give T as
     # one) has to become an array of that size

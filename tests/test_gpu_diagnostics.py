@@ -294,3 +294,39 @@ def test_sums_beyond_the_range_of_fp32(T, thermal):
         E = h.sum(0) / rho
         assert (np.abs(m["T"] - c * (E - uu / 2)) <= 2.0 ** -47 * c * (np.abs(h).sum(0) / rho + uu)).all()
     assert abs(again[6]) <= 2.0 ** -40 * uu.sum() and again[7] == d[7]  # (the snapshot is FP32)
+
+
+@pytest.mark.parametrize("what", ["moments", "populations"])
+def test_host_outputs_stay_as_they_are_until_the_queued_work_is_done(T, what):
+    # work queued earlier may still read an array that a call is about to overwrite in stream
+    # order: while a few tenths of a second of steps run, a call waiting behind them on another
+    # thread leaves every byte of its pageable outputs alone
+    import threading
+
+    import torch
+
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        lat = T.Lattice(*W.rayleigh_benard(512, 256, seed=69))
+        lat.step(100)
+        lat.moments(), lat.populations()
+        lat.step(60000)
+        done = torch.cuda.Event()
+        done.record(stream)
+    n = 512 * 256
+    arrays = [np.full(n, 1.0 / 3.0) for _ in range(4)] if what == "moments" else [np.full(9 * n, 1.0 / 3.0) for _ in range(2)]
+    call = (lambda: T.tclbm_moments(lat.handle, *[a.ctypes.data for a in arrays], 0)) if what == "moments" else \
+        (lambda: T.tclbm_get_populations(lat.handle, *[a.ctypes.data for a in arrays], 0))
+    thread = threading.Thread(target=call)
+    thread.start()
+    looks = 0
+    while True:
+        same = all((a == 1.0 / 3.0).all() for a in arrays)
+        if done.query():
+            break
+        assert same
+        looks += 1
+    thread.join()
+    assert looks > 3 and all((a != 1.0 / 3.0).all() for a in arrays)
+    assert np.array_equal(arrays[0], (lat.moments()["rho"] if what == "moments" else lat.populations()[0]).ravel())
+    lat.close()
