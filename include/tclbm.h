@@ -145,21 +145,22 @@ tclbm_status tclbm_init_fields(tclbm_lattice* lat, const double* rho, const doub
  * columns, a stream that is not capturing), the launches of one call are chained: each
  * work item of a launch waits only for the nine items around it in the previous launch,
  * so consecutive steps overlap on the device; the first launch of a call waits for
- * whatever precedes it on the stream.  The states are bit-identical to one step per call.  A chained wait that
- * expires is reported like the other bounded waits (TCLBM_ETIMEOUT at the next
- * synchronising call).
+ * whatever precedes it on the stream.  The states are bit-identical to one step per call.
+ * A chained wait that expires is reported like the other bounded waits (TCLBM_ETIMEOUT at
+ * the next synchronising call).
  *
  * A lattice small enough for the shared memory of the device (about 60,000 nodes with the
  * correction term, 190,000 without, 390,000 athermal; no work term) whose kernel and
- * launch shape are the library's choice takes 8 or more steps (12 or more where 2-D tiles are
- * its one-step kernel) in cooperative launches that
- * keep its state resident (up to 1024 steps each), unless the stream is capturing.  Such a
- * launch keeps the multiprocessors it uses to itself, so where handles of this process are on
- * more than one stream of the device only lattices that fit on it eight times over (2000
- * nodes or so with the correction term, 6000 athermal) run resident; the others then take one
- * launch per step, which share the device.  The states are the same bit for bit.  The first such call allocates, through the hooks, an
- * exchange board of 192 bytes per node (96 athermal); without it the lattice takes one
- * launch per step.  The bounded waits of these launches are reported in the same way. */
+ * launch shape are the library's choice takes 8 or more steps (12 or more where 2-D tiles
+ * are its one-step kernel) in cooperative launches that keep its state resident (up to 1024
+ * steps each), unless the stream is capturing.  Such a launch keeps the multiprocessors it
+ * uses to itself for up to a few milliseconds.  Where handles of this process are on more
+ * than one stream of the device, only lattices that fit on it eight times over (about 3,600
+ * nodes with the correction term, 7,000 athermal) run resident; the others then take one
+ * launch per step, which share the device.  The states are the same bit for bit.  The first
+ * resident call allocates, through the hooks, an exchange board of 192 bytes per node (96
+ * athermal); without it the lattice takes one launch per step.  The bounded waits of these
+ * launches are reported in the same way. */
 tclbm_status tclbm_step(tclbm_lattice* lat, int64_t nsteps);
 
 /* Macroscopic fields of the current state (Eq. 20; T per Section IV, T0 if athermal),
@@ -290,7 +291,8 @@ tclbm_status tclbm_set_tile(tclbm_lattice* lat, int32_t tx, int32_t ty);
  * library picks per lattice size: 0 above 2,097,152 nodes, and from 1,048,576 for thermal
  * lattices with the correction term, 512 or more columns, no work term and launches that
  * chain (up to 1,572,864 nodes, or up to 2,097,152 with a narrow last strip, calls of fewer
- * than 4 steps and captured calls run under 2 all the same); else 2 (or 1 where 2 does not apply).  Interior nodes evolve bit-identically under all variants; wall
+ * than 4 steps and captured calls run under 2 all the same); else 2 (or 1 where 2 does not
+ * apply).  Interior nodes evolve bit-identically under all variants; wall
  * nodes may differ in the last bit (multiply-add contraction).  Changing the variant
  * resets the launch shape to that variant's default.  EINVAL for other values. */
 tclbm_status tclbm_set_kernel(tclbm_lattice* lat, int32_t kind);

@@ -105,7 +105,9 @@ __device__ __forceinline__ void sum_add(Sum3& p, float v) {
     p.lo = __fadd_rn(p.lo, e);
 }
 // base + sum, for sums that are narrow()
-__device__ __forceinline__ double sum_value(double base, const Sum3& p) { return base + f2d(p.hi) + (f2d(p.mid) + f2d(p.lo)); }
+__device__ __forceinline__ double sum_value(double base, const Sum3& p) {
+    return base + f2d(p.hi) + (f2d(p.mid) + f2d(p.lo));
+}
 __device__ __forceinline__ double sum_value(const Sum3& p) { return f2d(p.hi) + (f2d(p.mid) + f2d(p.lo)); }
 template <int N>
 __device__ __forceinline__ Sum3 sum_of(const float (&v)[N]) {
@@ -177,7 +179,8 @@ template <bool THERMAL>
 __device__ __forceinline__ NodeTotals node_totals(const FieldParams& p, const NodeSums& s, const float (&f)[9],
                                                   const float (&h)[9]) {
     if (s.narrow())
-        return NodeTotals{sum_value(1.0, s.drho), sum_value(s.jx), sum_value(s.jy), THERMAL ? sum_value(p.hrest, s.sdh) : 0.0};
+        return NodeTotals{sum_value(1.0, s.drho), sum_value(s.jx), sum_value(s.jy),
+                          THERMAL ? sum_value(p.hrest, s.sdh) : 0.0};
     const int ex[9] = {0, 1, 0, -1, 0, 1, -1, -1, 1}, ey[9] = {0, 0, 1, 0, -1, 1, 1, -1, -1};
     NodeTotals t = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll

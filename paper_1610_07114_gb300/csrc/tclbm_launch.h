@@ -158,7 +158,8 @@ inline bool res_plan(const DevParams& p, int kind, int sms, ResPlan& best) {
         if (multi && kind == RES_CORR) continue;  // one launch per step of 2-D tiles is faster there (512 x 256: 5.9 against 7.1 us)
         // cells read from the board: columns beside the tile (and its corners), rows above and below
         const int cols = selfx ? 0 : 2 * R * (bh + 2 * R), rows = selfy ? 0 : 2 * R * bw;
-        const double cost = (multi ? 1.3 : 1.0) * (selfx || selfy ? 1.03 : 1.0) * own + 0.4 * halo + 0.15 * cols + 0.05 * rows;
+        const double cost = (multi ? 1.3 : 1.0) * (selfx || selfy ? 1.03 : 1.0) * own + 0.4 * halo + 0.15 * cols +
+                            0.05 * rows;
         if (cost < least) {
             least = cost;
             int threads = (own + halo + 31) / 32 * 32;
